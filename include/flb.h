@@ -127,7 +127,9 @@ int flb_sync(flb_lattice h);
 int flb_time(flb_lattice h, int64_t* t);
 
 /* Checkpoint and resume. A run continues exactly (the same noise draws, the
- * same sampling schedule, the same sums up to FP64 rounding order) from its
+ * same sampling schedule, the same sums up to FP64 rounding order --
+ * up to the rounding of the FP32 partials (FLB_OPT_PIPELINE_SAMPLING 3) where an
+ * FP32 run mixes calls of one or two steps with longer ones) from its
  * state f_i(x, t) (flb_get_populations), its time t (flb_time) and its raw
  * sums (flb_raw_sums): on a new handle with the same parameters call
  * flb_set_sampling (which clears the sums), then flb_set_raw_sums,
@@ -459,8 +461,10 @@ int flb_server_stats(flb_server s, flb_serve_stats* out);
 int flb_server_set_tile(flb_server s, int32_t tile);
 
 /* Tuning and testing options of a lattice handle.
- *  FLB_OPT_KERNEL: which step kernel runs -- FLB_KERNEL_AUTO (default: the
- *    pipelined TMA kernel for FP32, the generic kernel for FP64),
+ *  FLB_OPT_KERNEL: which step kernel runs -- FLB_KERNEL_AUTO (default: for FP32
+ *    the pipelined TMA kernel, or, in calls of three steps or more on lattices
+ *    that fit the SMs' shared memory, a kernel that makes all of them in one
+ *    launch; the generic kernel for FP64),
  *    FLB_KERNEL_GENERIC (one node per thread, plain loads) or
  *    FLB_KERNEL_PIPELINED (FP32 only). All give the same results up to rounding.
  *  FLB_OPT_PIPELINE_WARPS: colliding warps per CTA of the pipelined kernel

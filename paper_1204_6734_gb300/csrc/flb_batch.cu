@@ -113,15 +113,6 @@ int64_t replica_tiles(const flb_params& p, int tile) {
            ((p.Ly + tile_rows(tile) - 1) / tile_rows(tile));
 }
 
-int64_t count_sampled(int64_t ta, int64_t tb, int64_t warmup, int64_t every) {
-    if (every <= 0) return 0;
-    const int64_t lo = std::max(ta, warmup);
-    if (lo >= tb) return 0;
-    const int64_t first = warmup + (lo - warmup + every - 1) / every * every;
-    if (first >= tb) return 0;
-    return (tb - 1 - first) / every + 1;
-}
-
 int64_t slot_time(const flb_batch_s* b, const BatchSlot& s) {
     return std::min<int64_t>(b->step - s.join, s.tend);
 }

@@ -17,6 +17,7 @@
 #include "flb_io.cuh"
 #include "flb_structure.h"
 #include "flb_kernels.cuh"
+#include "flb_resident.cuh"
 
 namespace flb {
 
@@ -285,6 +286,11 @@ struct flb_lattice_s {
     int variant;           // FLB_KERNEL_*
     TmaPlan tma;           // pipelined FP32 kernel (tensor maps, launch shape)
     TmaPlan tma_quiet;     // the same for steps without sampling, when it differs
+    // many steps per launch with the state on the SMs (FP32, flb_resident.cuh)
+    ResidentPlan res;
+    uint64_t* mail = nullptr;        // the blocks' mailboxes (two), when the lattice is cut
+    uint32_t tag = 0;                // steps that resident launches made so far
+    bool one_step = false;           // an option chose the one-step kernel's shape
     const float* lut32 = nullptr;    // velocity tables (look-up-table f-norm)
     const double* lut64 = nullptr;
     double ref[9];
@@ -394,6 +400,70 @@ cudaError_t launch_step_tma(flb_lattice h, bool sample, float* fields) {
     return tma_step(plan, h->cur, a, collide_const<float>(&h->p), h->p.basis, sample, h->stream);
 }
 
+// How many of the next n steps one resident launch takes (0: none): the kernel
+// is on, the lattice fits, and the stream is not being captured (a mailbox tag
+// may not be replayed). The steps before the first sampled one go by themselves
+// (the kernel without sampling) where that leaves no short launch.
+int64_t resident_steps(flb_lattice h, int64_t n) {
+    if (!h->res.gx || h->variant != FLB_KERNEL_AUTO || h->one_step || h->slab) return 0;
+    n = std::min<int64_t>(n, kResMaxSteps);
+    if (n < kResMinSteps) return 0;
+    if (h->every > 0 && h->t < h->warmup) {
+        const int64_t quiet = h->warmup - h->t;
+        if (quiet >= kResMinSteps && n - quiet >= kResMinSteps) n = quiet;
+    }
+    if (count_sampled(h->t, h->t + n, h->warmup, h->every) > 0 &&
+        (!h->res.smem[1] || h->tma.sample_mode != kPlanTensorSampling))
+        return 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return cap == cudaStreamCaptureStatusNone ? n : 0;
+}
+
+cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
+    ResidentArgs a;
+    std::memset((void*)&a, 0, sizeof(a));
+    const int64_t ns = count_sampled(h->t, h->t + n, h->warmup, h->every);
+    a.k.src = (const float*)h->buf[h->cur];
+    a.k.dst = (float*)h->buf[h->cur ^ (n & 1)];
+    a.k.geo = h->geo;
+    a.k.gx = h->res.gx;
+    a.k.gy = h->res.gy;
+    a.k.mail = h->mail;
+    a.k.mail_words = (int)h->res.mail_words;
+    a.k.tag0 = h->tag;
+    a.k.t0 = (uint32_t)h->t;
+    a.k.n = n;
+    a.k.first = n;
+    a.k.every = 1;
+    if (ns > 0) {
+        const int64_t since = h->t - h->warmup;
+        a.k.first = (int)(since < 0 ? -since : (h->every - since % h->every) % h->every);
+        a.k.every = (int)std::min<int64_t>(h->every, kResMaxSteps);
+    }
+    a.k.acc = h->acc;
+    a.k.err = h->err;
+    a.k.lut = h->lut32;
+    a.k.fields = fields;
+    a.s = tensor_sampling_ok(&h->p) ? gram_scale(&h->p) : 1.0;
+    a.sinv = (float)(1.0 / a.s);
+    for (int i = 0; i < 9; ++i) {
+        a.ref[i] = (float)h->ref[i];
+        a.snref[i] = (float)(-h->ref[i] / a.s);
+    }
+    const cudaError_t ce = resident_step(h->res, a, collide_const<float>(&h->p), h->p.basis, ns > 0, h->stream);
+    if (ce == cudaSuccess) {
+        h->tag += (uint32_t)n;
+        h->nsamp += ns * (int64_t)h->p.Lx * h->p.Ly;
+        h->t += n;
+        h->cur ^= n & 1;
+    }
+    return ce;
+}
+
 bool uses_tma(flb_lattice h) {
     return h->p.precision == FLB_FP32 && h->variant != FLB_KERNEL_GENERIC;
 }
@@ -472,15 +542,35 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
         }
         h->ws = (char*)dev_workspace;
         h->own_ws = false;
+        if (p->precision == FLB_FP32) h->res = resident_plan(p->Lx, p->Ly, sms, false);
     } else {
+        // the mailboxes of a cut lattice are part of the library's own
+        // allocation (a caller's workspace keeps its size: the lattice is then
+        // not cut)
+        if (p->precision == FLB_FP32) h->res = resident_plan(p->Lx, p->Ly, sms, true);
+        const size_t mail = 2 * sizeof(uint64_t) * (size_t)h->res.mail_words;
         void* ptr = nullptr;
-        if (cudaMalloc(&ptr, L.total) != cudaSuccess) {
+        if (mail && cudaMalloc(&ptr, L.total + mail) != cudaSuccess) {
+            cudaGetLastError();
+            ptr = nullptr;
+            h->res = resident_plan(p->Lx, p->Ly, sms, false);
+        }
+        if (!ptr && cudaMalloc(&ptr, L.total) != cudaSuccess) {
             cudaGetLastError();
             delete h;
             return FLB_ERR_OOM;
         }
         h->ws = (char*)ptr;
         h->own_ws = true;
+        if (h->res.mail_words) {
+            h->mail = (uint64_t*)(h->ws + L.total);
+            if (cudaMemsetAsync(h->mail, 0, mail, stream) != cudaSuccess) {
+                cudaGetLastError();
+                cudaFree(ptr);
+                delete h;
+                return FLB_ERR_CUDA;
+            }
+        }
     }
     h->ws_bytes = L.total;
     h->buf[0] = h->ws;
@@ -536,6 +626,10 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
             cudaGetLastError();
             h->tma_quiet.ready = false;
         }
+    }
+    if (ce == cudaSuccess && h->res.gx && resident_prepare(h->res, p->basis) != cudaSuccess) {
+        cudaGetLastError();
+        h->res.gx = 0;
     }
     if (ce == cudaSuccess && p->precision == FLB_FP16_DEV)
         ce = fp16_plan(&h->tma, h->buf[0], h->buf[1], h->geo);
@@ -711,7 +805,7 @@ int flb_step(flb_lattice h, int64_t n) {
     if (!h || n < 0) return FLB_ERR_ARG;
     if (h->sticky) return h->sticky;
     const long long N = (long long)h->p.Lx * h->p.Ly;
-    for (int64_t s = 0; s < n; ++s) {
+    for (int64_t s = 0; s < n;) {
         const bool sample =
             h->every > 0 && h->t >= h->warmup && ((h->t - h->warmup) % h->every) == 0;
         cudaError_t ce = cudaSuccess;
@@ -724,6 +818,27 @@ int flb_step(flb_lattice h, int64_t n) {
         if (sk_due && !fields)
             ce = structure_sample(h->sk, h->buf[h->cur], h->p.precision, h->geo, dev_codec(h), h->ref,
                                   h->stream);
+        // up to the next structure-factor sample in one launch
+        int64_t run = n - s;
+        if (h->sk_every > 0) {
+            const int64_t next = h->t < h->sk_warmup ? h->sk_warmup
+                                                     : h->t + h->sk_every - (h->t - h->sk_warmup) % h->sk_every;
+            run = std::min(run, next - h->t);
+        }
+        run = ce == cudaSuccess ? resident_steps(h, run) : 0;
+        if (run > 0) {
+            ce = launch_resident(h, (int)run, fields);
+            if (ce == cudaSuccess) {
+                s += run;
+                if (fields) ce = structure_sample_fields(h->sk, h->stream);
+                if (ce != cudaSuccess) return FLB_ERR_CUDA;
+                continue;
+            }
+            if (ce != cudaErrorCooperativeLaunchTooLarge) return FLB_ERR_CUDA;
+            cudaGetLastError();   // SMs not all available to this process: one step per launch
+            h->res.gx = 0;
+            ce = cudaSuccess;
+        }
         if (ce == cudaSuccess) ce = launch_step(h, sample, fields);
         if (ce == cudaSuccess && fields) ce = structure_sample_fields(h->sk, h->stream);
         if (ce == cudaSuccess && sample && !reduces_in_kernel(h)) {
@@ -735,6 +850,7 @@ int flb_step(flb_lattice h, int64_t n) {
         if (ce != cudaSuccess) return FLB_ERR_CUDA;
         h->t += 1;
         h->cur ^= 1;
+        ++s;
     }
     return FLB_OK;
 }
@@ -766,6 +882,7 @@ int flb_set_option(flb_lattice h, int32_t option, int32_t value) {
             return FLB_ERR_ARG;
         }
         h->tma = plan;
+        h->one_step = true;
         return FLB_OK;
     }
     if (option == FLB_OPT_PIPELINE_WARPS) {
@@ -780,6 +897,7 @@ int flb_set_option(flb_lattice h, int32_t option, int32_t value) {
         if (plan.sample_mode == kPlanTensorSampling && !tensor_sampling_ok(&h->p)) return FLB_ERR_ARG;
         h->tma = plan;
         h->tma_quiet.ready = false;   // the given count for every step
+        h->one_step = true;
         return FLB_OK;
     }
     return FLB_ERR_ARG;

@@ -122,6 +122,65 @@ __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
     gram_step<3>(g.ld, c);
 }
 
+// The same sums from deviations staged as two FP16 numbers, h + l with l the
+// rounding error of h rounded again: 22 bits of a value, so that the products
+// h h + h l + l h carry FP32's accuracy (l l, below 2^-22 of them, is left out).
+// The l block has the layout of the h block, its row 9 zero; the three products
+// share the FP32 accumulators.
+__device__ __forceinline__ void gram_zero_row(__half* blk) {
+    reinterpret_cast<uint32_t*>(blk)[9 * (kGramRowHalves / 2) + (threadIdx.x & 31)] = 0u;
+}
+
+template <int I>
+__device__ __forceinline__ void gram_store_pair(uint32_t st, uint32_t sl, f2 h) {
+    const __half2 v = __floats2half2_rn(h.v.x, h.v.y);
+    const float2 b = __half22float2(v);
+    const f2 d = h - f2(b);
+    const __half2 w = __floats2half2_rn(d.v.x, d.v.y);
+    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(st), "n"(2 * kGramRowHalves * I),
+                 "r"(*reinterpret_cast<const uint32_t*>(&v)));
+    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(sl), "n"(2 * kGramRowHalves * I),
+                 "r"(*reinterpret_cast<const uint32_t*>(&w)));
+}
+
+__device__ __forceinline__ void gram_stage_pair(const GramLane& g, const GramLane& l, const f2 (&h)[9]) {
+    __syncwarp();
+    gram_store_pair<0>(g.st, l.st, h[0]);
+    gram_store_pair<1>(g.st, l.st, h[1]);
+    gram_store_pair<2>(g.st, l.st, h[2]);
+    gram_store_pair<3>(g.st, l.st, h[3]);
+    gram_store_pair<4>(g.st, l.st, h[4]);
+    gram_store_pair<5>(g.st, l.st, h[5]);
+    gram_store_pair<6>(g.st, l.st, h[6]);
+    gram_store_pair<7>(g.st, l.st, h[7]);
+    gram_store_pair<8>(g.st, l.st, h[8]);
+}
+
+template <int S>
+__device__ __forceinline__ void gram_step_pair(uint32_t ld, uint32_t ll, float (&c)[8]) {
+    uint32_t d0, d1, d2, d3, e0, e1, e2, e3;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4+%5];"
+                 : "=r"(d0), "=r"(d1), "=r"(d2), "=r"(d3)
+                 : "r"(ld), "n"(32 * S));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4+%5];"
+                 : "=r"(e0), "=r"(e1), "=r"(e2), "=r"(e3)
+                 : "r"(ll), "n"(32 * S));
+    mma16816(c, 0, d0, d1, d2, d3, d0, d2);
+    mma16816(c, 4, d0, d1, d2, d3, d1, d3);
+    mma16816(c, 0, d0, d1, d2, d3, e0, e2);
+    mma16816(c, 4, d0, d1, d2, d3, e1, e3);
+    mma16816(c, 0, e0, e1, e2, e3, d0, d2);
+    mma16816(c, 4, e0, e1, e2, e3, d1, d3);
+}
+
+__device__ __forceinline__ void gram_mma_pair(const GramLane& g, const GramLane& l, float (&c)[8]) {
+    __syncwarp();
+    gram_step_pair<0>(g.ld, l.ld, c);
+    gram_step_pair<1>(g.ld, l.ld, c);
+    gram_step_pair<2>(g.ld, l.ld, c);
+    gram_step_pair<3>(g.ld, l.ld, c);
+}
+
 // Add the FP32 partials to the FP64 matrix cm[16][16] (rows and columns 0..9
 // only) and clear them. Fragment of thread (g, q) = (lane / 4, lane % 4):
 // c[0..3] = C[g][2q], C[g][2q+1], C[g+8][2q], C[g+8][2q+1]; c[4..7] the same

@@ -73,6 +73,16 @@ inline bool tensor_sampling_ok(const flb_params* p) {
 }
 inline double gram_scale(const flb_params* p) { return std::sqrt(p->kT * p->rho0); }
 
+// Steps of [ta, tb) that the schedule (warmup, every) samples.
+inline int64_t count_sampled(int64_t ta, int64_t tb, int64_t warmup, int64_t every) {
+    if (every <= 0) return 0;
+    const int64_t lo = ta > warmup ? ta : warmup;
+    if (lo >= tb) return 0;
+    const int64_t first = warmup + (lo - warmup + every - 1) / every * every;
+    if (first >= tb) return 0;
+    return (tb - 1 - first) / every + 1;
+}
+
 inline int grid_for(long long n) {
     long long b = (n + 255) / 256;
     if (b > 4096) b = 4096;

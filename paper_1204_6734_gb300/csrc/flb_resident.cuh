@@ -1,0 +1,530 @@
+// flb_resident.cuh -- many time steps per launch of an FP32 lattice whose
+// populations stay in shared memory between the steps.
+//
+// The lattice is cut into gx x gy blocks, one CTA each (one block: the whole
+// lattice in one CTA). A CTA loads the pre-collision populations of its nodes
+// once, steps them n times and stores the result once, in the ghost-frame
+// layout of every other kernel. Against one launch per step this saves the
+// launch, the pipeline's start and its end in every step (7 to 9 us of the
+// 8.1 us that a step of a 21 x 21 lattice took, of 10 us at 300 x 130 and of
+// 20 us at 1000 x 750) and the trip of 72 bytes per node through L2 or HBM.
+//
+// In place: one copy of the populations, cell (X, Y, i) at (X + bw Y) 9 + i
+// (stride 9 words: no bank conflicts). s steps after the load, f_i of node
+// (x, y) sits in cell ((x - s v_ix) mod bw, (y - s v_iy) mod bh): the node
+// reads its nine cells, collides and writes f*_i back to the same nine cells,
+// and because the offsets have moved on by one, the next step's read of node
+// x + v_i is that cell. Streaming costs no copy, no cell is touched by two
+// threads in a step, one barrier per step orders the steps, and the wrap of
+// the offsets is the periodic boundary where the lattice is not cut.
+//
+// Node pairs (packed FP32x2): node A is the m-th of the block, node B the m-th
+// from its end, i.e. (bw - 1 - x, bh - 1 - y), so B's cells follow from A's
+// by one subtraction each (cell_i(B) = nn - 1 - cell_opposite(i)(A)), and the
+// block's first and last row are done first, in the same pass: what they send
+// is under way while the rows between them are computed.
+//
+// Between blocks: a population that leaves its block is written, besides, to a
+// mailbox in global memory as one 64-bit word {value, tag}, tag = a number
+// that grows with every step and launch of the handle. The reader polls the
+// word itself until the tag is the one of its step: one trip through L2, no
+// fence and no flag. Two mailboxes alternate; a word of one is overwritten
+// two steps later, by a node that has by then received the populations of the
+// very nodes that read it, so no reader can be overtaken. All CTAs are
+// resident at once (cooperative launch), every wait is bounded (flb_tma.cuh).
+//
+// Correlation sums: as flb_gram.cuh, except that every step's FP32 partials
+// (at most 1024 products per warp, added over the CTA's warps in FP32 in a
+// fixed order) go to FP64 by themselves: the sums do not depend on how many
+// steps a launch makes. Where a batch's tile shape promises FP32 products, the
+// deviations are staged as two FP16 numbers (h + l, 22 bits) and the products
+// are h h + h l + l h, all exact in the FP32 accumulator's inputs.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "flb_collide.cuh"
+#include "flb_gram.cuh"
+#include "flb_kernels.cuh"
+#include "flb_pipeline.cuh"
+#include "flb_layout.cuh"
+#include "flb_tma.cuh"
+
+namespace flb {
+
+constexpr int kResMaxWarps = 16;   // 512 threads of 128 registers
+constexpr int kResEntries = 84;    // Gram entries kept: rows 0..7 x columns 0..9, rows 8, 9 x 8, 9
+constexpr int kResSlot = 96;       // floats per warp and parity
+
+// Sampling of a resident launch: none; deviations staged in FP16; FP32 products.
+enum : int { kResQuiet = 0, kResStaged = 1, kResExact = 2 };
+
+__host__ __device__ constexpr size_t res_cells_bytes(int cells) { return ((size_t)cells * 36 + 15) / 16 * 16; }
+__host__ __device__ constexpr size_t res_sample_bytes(int mode, int warps) {
+    return mode == kResQuiet ? 0
+                             : (size_t)warps * ((mode == kResExact ? 2 : 1) * kGramWarpHalves * 2 + 2 * kResSlot * 4) +
+                                   kResSlot * 8;
+}
+// Dynamic shared memory of a CTA of `warps` warps holding `cells` nodes.
+__host__ __device__ constexpr size_t res_smem_bytes(int cells, int mode, int warps) {
+    return res_cells_bytes(cells) + res_sample_bytes(mode, warps) + 16;
+}
+
+// One CTA's block of one lattice and what to do with it.
+struct ResBlock {
+    const float* src;       // holds f*(t0 - 1)
+    float* dst;             // receives f*(t0 + n - 1)
+    Geometry geo;
+    int x0, y0, bw, bh;
+    int gx, gy, ix, iy;     // the block's place in the grid of blocks
+    uint64_t* mail;         // two mailboxes of mail_words words (gx gy > 1)
+    int mail_words;
+    uint32_t tag0;          // tag of the state at t0
+    uint32_t t0;
+    int n;
+    int first, every;       // steps of this launch sampled: first, first + every, ...
+    double* acc;
+    DevError* err;
+    const float* lut;
+    float* fields;          // structure-factor fields of the state at t0 (or null)
+};
+
+__device__ __forceinline__ uint64_t ld_mail(const uint64_t* p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_mail(uint64_t* p, float v, uint32_t tag) {
+    const uint64_t w = (uint64_t)tag << 32 | __float_as_uint(v);
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+
+// Place of population i among the three that cross a y (x) boundary together.
+__host__ __device__ constexpr int res_ky(int i) { return i == 2 || i == 4 ? 0 : (i == 5 || i == 7 ? 1 : 2); }
+__host__ __device__ constexpr int res_kx(int i) { return i == 1 || i == 3 ? 0 : (i == 5 || i == 6 ? 1 : 2); }
+__host__ __device__ constexpr int opposite(int i) { return i == 0 ? 0 : (i < 5 ? (i + 1) % 4 + 1 : (i - 3) % 4 + 5); }
+static_assert(opposite(1) == 3 && opposite(2) == 4 && opposite(3) == 1 && opposite(4) == 2 && opposite(5) == 7 &&
+                  opposite(6) == 8 && opposite(7) == 5 && opposite(8) == 6,
+              "opposite velocities");
+
+// Words of one mailbox: the y boundaries (upwards, downwards), Lx columns of
+// three populations each, then the x boundaries, Ly rows.
+inline long long res_mail_words(int Lx, int Ly, int gx, int gy) {
+    return (gy > 1 ? 6LL * gy * Lx : 0) + (gx > 1 ? 6LL * gx * Ly : 0);
+}
+
+// Which edges of its block node A of a pair lies on (only edges where the
+// lattice is cut). Node B, the pair's image, lies on the opposite ones and
+// exchanges the opposite populations there.
+struct ResEdge {
+    bool l, r, b, t;
+    __device__ __forceinline__ bool any() const { return l || r || b || t; }
+};
+
+// Mailbox word of population I pulled by (In) or leaving from (!In) node (X, Y)
+// across a y boundary (AXIS 1) or an x boundary (AXIS 0). The word belongs to
+// the sender: the direction, the sender's row (column) of blocks, the
+// population, the sender's X (Y).
+template <int AXIS, int I, bool In>
+__device__ __forceinline__ int res_word(const ResBlock& k, int X, int Y) {
+    if constexpr (AXIS == 1) {
+        const int j = In ? wrap(k.iy - cvy(I), k.gy) : k.iy;
+        return (((cvy(I) > 0 ? 0 : k.gy) + j) * 3 + res_ky(I)) * k.geo.Lx + (In ? wrap(X - cvx(I), k.geo.Lx) : X);
+    } else {
+        const int j = In ? wrap(k.ix - cvx(I), k.gx) : k.ix, y0 = k.gy > 1 ? 6 * k.gy * k.geo.Lx : 0;
+        return y0 + (((cvx(I) > 0 ? 0 : k.gx) + j) * 3 + res_kx(I)) * k.geo.Ly + (In ? wrap(Y - cvy(I), k.geo.Ly) : Y);
+    }
+}
+
+// The nine cells of node A (word offsets, without the population's own offset)
+// from its row and column offsets, and node B's from them.
+struct ResCells {
+    int r[3], c[3];   // index v + 1
+    int kb;           // 9 (nn - 1)
+    __device__ __forceinline__ int a(int i) const { return r[cvy(i) + 1] + c[cvx(i) + 1] + i; }
+    __device__ __forceinline__ int b(int i) const {
+        return kb - (r[1 - cvy(i)] + c[1 - cvx(i)]) + i;
+    }
+};
+
+// Receive across one edge: A's populations I0, I1, I2 and B's opposite ones,
+// into the pair's own cells, once all carry the step's tag. skip1, skip2: I1,
+// I2 cross the other axis' boundary, too, and came from there.
+template <int AXIS, int I0, int I1, int I2>
+__device__ __noinline__ void res_receive(const ResBlock& k, const uint64_t* in, uint32_t tag, uint32_t t, int X, int Y,
+                                         int XB, int YB, float* cell, const ResCells& a, bool skip1, bool skip2,
+                                         volatile int* gave_up) {
+    const uint64_t* pa0 = in + res_word<AXIS, I0, true>(k, X, Y);
+    const uint64_t* pa1 = in + res_word<AXIS, I1, true>(k, X, Y);
+    const uint64_t* pa2 = in + res_word<AXIS, I2, true>(k, X, Y);
+    const uint64_t* pb0 = in + res_word<AXIS, opposite(I0), true>(k, XB, YB);
+    const uint64_t* pb1 = in + res_word<AXIS, opposite(I1), true>(k, XB, YB);
+    const uint64_t* pb2 = in + res_word<AXIS, opposite(I2), true>(k, XB, YB);
+    const uint64_t have = (uint64_t)tag << 32;
+    uint64_t a0, a1 = have, a2 = have, b0, b1 = have, b2 = have;
+    long long began = 0;
+    while (true) {
+        a0 = ld_mail(pa0);
+        b0 = ld_mail(pb0);
+        if (!skip1) {
+            a1 = ld_mail(pa1);
+            b1 = ld_mail(pb1);
+        }
+        if (!skip2) {
+            a2 = ld_mail(pa2);
+            b2 = ld_mail(pb2);
+        }
+        const uint32_t bad = ((uint32_t)(a0 >> 32) ^ tag) | ((uint32_t)(b0 >> 32) ^ tag) | ((uint32_t)(a1 >> 32) ^ tag) |
+                             ((uint32_t)(b1 >> 32) ^ tag) | ((uint32_t)(a2 >> 32) ^ tag) | ((uint32_t)(b2 >> 32) ^ tag);
+        if (bad == 0 || *gave_up) break;
+        if (began == 0) {
+            began = clock64();
+        } else if (clock64() - began > kWaitCycles) {
+            record_error(k.err, kStatusTimeout, -1, t);
+            *gave_up = 1;
+            break;
+        }
+    }
+    cell[a.a(I0)] = __uint_as_float((uint32_t)a0);
+    cell[a.b(opposite(I0))] = __uint_as_float((uint32_t)b0);
+    if (!skip1) {
+        cell[a.a(I1)] = __uint_as_float((uint32_t)a1);
+        cell[a.b(opposite(I1))] = __uint_as_float((uint32_t)b1);
+    }
+    if (!skip2) {
+        cell[a.a(I2)] = __uint_as_float((uint32_t)a2);
+        cell[a.b(opposite(I2))] = __uint_as_float((uint32_t)b2);
+    }
+}
+
+// Send across one edge: A's populations I0, I1, I2 and (unless B is A) B's
+// opposite ones, read back from the pair's cells.
+template <int AXIS, int I0, int I1, int I2>
+__device__ __noinline__ void res_send(const ResBlock& k, uint64_t* out, uint32_t tag, int X, int Y, int XB, int YB,
+                                      const float* cell, const ResCells& a, bool skip1, bool skip2, bool both) {
+    st_mail(out + res_word<AXIS, I0, false>(k, X, Y), cell[a.a(I0)], tag);
+    if (!skip1) st_mail(out + res_word<AXIS, I1, false>(k, X, Y), cell[a.a(I1)], tag);
+    if (!skip2) st_mail(out + res_word<AXIS, I2, false>(k, X, Y), cell[a.a(I2)], tag);
+    if (!both) return;
+    st_mail(out + res_word<AXIS, opposite(I0), false>(k, XB, YB), cell[a.b(opposite(I0))], tag);
+    if (!skip1) st_mail(out + res_word<AXIS, opposite(I1), false>(k, XB, YB), cell[a.b(opposite(I1))], tag);
+    if (!skip2) st_mail(out + res_word<AXIS, opposite(I2), false>(k, XB, YB), cell[a.b(opposite(I2))], tag);
+}
+
+// A warp's FP32 partials of one step, in the order of the kept entries (C is
+// symmetric): rows 0..7 by columns 0..7, rows 0..7 by columns 8 and 9, rows 8
+// and 9 by columns 8 and 9. Cleared for the next sampled step.
+__device__ __forceinline__ void res_publish(float (&c)[8], float* slot) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    *reinterpret_cast<float2*>(slot + 2 * lane) = make_float2(c[0], c[1]);
+    if (q == 0) {
+        *reinterpret_cast<float2*>(slot + 64 + 2 * g) = make_float2(c[4], c[5]);
+        if (g < 2) *reinterpret_cast<float2*>(slot + 80 + 2 * g) = make_float2(c[6], c[7]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) c[i] = 0.f;
+}
+
+// The CTA's sum of a step's partials of nw warps, added to the FP64 entries by
+// the last 96 threads of the CTA (warps without nodes of their own where the
+// block leaves room for them; entry q always by the same thread). All loads are
+// under way before the first add: this sits in the step's critical path.
+__device__ __forceinline__ void res_reduce(const float* slots, double* red, int nw) {
+    const int T = blockDim.x, r0 = T > kResSlot ? T - kResSlot : 0;
+    for (int q = (int)threadIdx.x - r0; q >= 0 && q < kResEntries; q += T) {
+        float v[kResMaxWarps];
+#pragma unroll
+        for (int w = 0; w < kResMaxWarps; ++w) v[w] = w < nw ? slots[w * kResSlot + q] : 0.f;
+#pragma unroll
+        for (int h = kResMaxWarps / 2; h > 0; h >>= 1)
+#pragma unroll
+            for (int w = 0; w < h; ++w) v[w] += v[w + h];
+        red[q] += (double)v[0];
+    }
+}
+
+// Sum q of the kSums layout from the kept entries.
+__device__ __forceinline__ double res_sum(const double* red, int q, double s) {
+    if (q < 9) return s * red[q < 8 ? 64 + 2 * q + 1 : 81];
+    int k = q - 9, i = 0;
+    while (k >= 9 - i) {
+        k -= 9 - i;
+        ++i;
+    }
+    const int j = i + k;
+    return s * s * red[j < 8 ? 8 * i + j : (i < 8 ? 64 + 2 * i : 80)];
+}
+
+// Steps 0..n-1 of one block. Par: the lattice's parameters -- key, cc (the
+// collision constants), s (the Gram scale), scaled(f, i) (the deviation of
+// population i in units of s), ref(i) (f_i^0(rho0, u0)).
+template <int BASIS, int SAMPLE, class Par>
+__device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, unsigned char* smem) {
+    float* cell = reinterpret_cast<float*>(smem);
+    const int T = blockDim.x, c = threadIdx.x, lane_id = c & 31, warp = c >> 5, nw = T >> 5;
+    const int bw = k.bw, bh = k.bh, nn = bw * bh, pairs = (nn + 1) >> 1;
+    const int nwork = min(nw, (pairs + 31) >> 5);   // warps with nodes
+    const int Lx = k.geo.Lx;
+    unsigned char* after = smem + res_cells_bytes(nn);
+    double* red = reinterpret_cast<double*>(after);
+    float* slots = reinterpret_cast<float*>(after + (SAMPLE ? kResSlot * 8 : 0));
+    __half* gram = reinterpret_cast<__half*>(slots + (SAMPLE ? 2 * nw * kResSlot : 0));
+    volatile int* gave_up =
+        reinterpret_cast<volatile int*>(after + res_sample_bytes(SAMPLE, nw));
+    if (c == 0) *gave_up = 0;
+
+    constexpr int kBlocks = SAMPLE == kResExact ? 2 : 1;
+    __half* blk = gram + warp * kBlocks * kGramWarpHalves;
+    const GramLane gh(SAMPLE ? smem_u32(blk) : 0u, kGramRows);
+    const GramLane gl(SAMPLE == kResExact ? smem_u32(blk + kGramWarpHalves) : 0u, kGramRows);
+    float gc[SAMPLE ? 8 : 1];
+    if constexpr (SAMPLE != kResQuiet) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) gc[q] = 0.f;
+        gram_init(blk);
+        if constexpr (SAMPLE == kResExact) gram_zero_row(blk + kGramWarpHalves);
+        for (int q = c - (T > kResSlot ? T - kResSlot : 0); q >= 0 && q < kResEntries; q += T) red[q] = 0.0;
+    }
+
+    // this thread's nodes: pairs c, c + T, ...
+    const int dy = T / bw, dx = T - dy * bw;
+    const int ys = c / bw, xs = c - ys * bw;
+    const bool cutx = k.gx > 1, cuty = k.gy > 1;
+    {
+        int x = xs, y = ys;
+        for (int m = c; m < pairs; m += T) {
+            const int X = k.x0 + x, Y = k.y0 + y, XB = k.x0 + bw - 1 - x, YB = k.y0 + bh - 1 - y;
+            float va[9], vb[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                va[i] = k.src[pull_at(k.geo, i, X, Y)];
+                vb[i] = k.src[pull_at(k.geo, i, XB, YB)];
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                cell[9 * m + i] = va[i];
+                cell[9 * (nn - 1 - m) + i] = vb[i];
+            }
+            x += dx;
+            y += dy;
+            if (x >= bw) {
+                x -= bw;
+                ++y;
+            }
+        }
+    }
+
+    int sx = 0, sy = 0;              // steps so far modulo bw, bh
+    int until = k.first;             // next step to sample
+    int nsum = 0;                    // sampled steps so far
+    bool pending = false;            // the previous step's partials wait in the slots
+    for (int st = 0; st < k.n; ++st) {
+        const uint32_t t = k.t0 + (uint32_t)st;
+        const bool last = st == k.n - 1;
+        const bool smp = SAMPLE != kResQuiet && st == until;
+        if (smp) until = k.every > k.n - st ? k.n : st + k.every;
+        if constexpr (SAMPLE != kResQuiet) {
+            if (pending) res_reduce(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
+            pending = false;
+        }
+        const uint64_t* in = k.mail + (size_t)(st & 1) * k.mail_words;
+        uint64_t* out = k.mail + (size_t)((st + 1) & 1) * k.mail_words;
+        int x = xs, y = ys;
+        for (int m0 = warp * 32; m0 < pairs; m0 += T) {
+            const int m = m0 + lane_id;
+            const bool inA = m < pairs, inB = inA && 2 * m != nn - 1;
+            ResCells a;
+            {
+                int cp = x - sx, cm = x + sx, rp = y - sy, rm = y + sy;
+                cp += cp < 0 ? bw : 0;
+                cm -= cm >= bw ? bw : 0;
+                rp += rp < 0 ? bh : 0;
+                rm -= rm >= bh ? bh : 0;
+                a.c[0] = 9 * cm;
+                a.c[1] = 9 * x;
+                a.c[2] = 9 * cp;
+                a.r[0] = 9 * bw * rm;
+                a.r[1] = 9 * bw * y;
+                a.r[2] = 9 * bw * rp;
+                a.kb = 9 * (nn - 1);
+            }
+            const int X = k.x0 + x, Y = k.y0 + y, XB = k.x0 + bw - 1 - x, YB = k.y0 + bh - 1 - y;
+            const ResEdge e{cutx && x == 0, cutx && x == bw - 1, cuty && y == 0, cuty && y == bh - 1};
+            const bool edge = inA && e.any();
+            if (edge && st > 0) {   // what comes across the cut: into this thread's own cells
+                const uint32_t tag = k.tag0 + (uint32_t)st;
+                if (e.b) res_receive<1, 2, 5, 6>(k, in, tag, t, X, Y, XB, YB, cell, a, false, false, gave_up);
+                if (e.t) res_receive<1, 4, 7, 8>(k, in, tag, t, X, Y, XB, YB, cell, a, false, false, gave_up);
+                if (e.l) res_receive<0, 1, 5, 8>(k, in, tag, t, X, Y, XB, YB, cell, a, e.b, e.t, gave_up);
+                if (e.r) res_receive<0, 3, 7, 6>(k, in, tag, t, X, Y, XB, YB, cell, a, e.t, e.b, gave_up);
+            }
+            auto load = [&](f2* g) {
+                if (inA) {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) g[i] = f2(cell[a.a(i)], cell[a.b(i)]);
+                } else {   // a lane past the end: any valid state
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) g[i] = f2(1.f);
+                }
+            };
+            f2 g[9];
+            load(g);
+            if (k.fields && st == 0) {
+                f2 d[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) d[i] = g[i] - f2(par.ref(i));
+                const f2 fr = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])) + d[8];
+                const f2 fx = (d[1] - d[3]) + ((d[5] - d[6]) + (d[8] - d[7]));
+                const f2 fy = (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
+                const size_t N = (size_t)Lx * k.geo.Ly;
+                if (inA) {
+                    float* o = k.fields + (size_t)Y * Lx + X;
+                    o[0] = fr.v.x;
+                    o[N] = fx.v.x;
+                    o[2 * N] = fy.v.x;
+                }
+                if (inB) {
+                    float* o = k.fields + (size_t)YB * Lx + XB;
+                    o[0] = fr.v.y;
+                    o[N] = fx.v.y;
+                    o[2 * N] = fy.v.y;
+                }
+            }
+            const uint32_t nodeA = (uint32_t)X + (uint32_t)Lx * (uint32_t)Y;
+            const uint32_t nodeB = (uint32_t)XB + (uint32_t)Lx * (uint32_t)YB;
+            auto refetch = [&](f2* gg) {
+                load(gg);
+                if constexpr (SAMPLE != kResQuiet) {
+                    if (smp) {
+                        f2 h[9];
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) {
+                            h[i] = par.scaled(gg[i], i);
+                            if (!inB) h[i] = f2(inA ? h[i].v.x : 0.f, 0.f);
+                        }
+                        if constexpr (SAMPLE == kResExact)
+                            gram_stage_pair(gh, gl, h);
+                        else
+                            gram_stage(gh, h);
+                    }
+                }
+            };
+            f2 f[9];
+            const uint32_t stt =
+                collide_basis<f2, BASIS>(g, PairNoise{par.key, nodeA, nodeB, t}, refetch, k.lut, par.cc, f);
+            if (stt) {
+                if (inA && (stt & 0xFF)) record_error(k.err, (int)(stt & 0xFF), nodeA, t);
+                if (inB && (stt >> 8)) record_error(k.err, (int)(stt >> 8), nodeB, t);
+            }
+            if (last) {
+                if (inA) store_lane_ghosts(k.dst + at(k.geo, 0, X, Y), k.geo, X, Y, f, 0);
+                if (inB) store_lane_ghosts(k.dst + at(k.geo, 0, XB, YB), k.geo, XB, YB, f, 1);
+            } else if (inA) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) cell[a.a(i)] = f[i].v.x;
+                if (inB)
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) cell[a.b(i)] = f[i].v.y;
+                if (edge) {
+                    const uint32_t tag = k.tag0 + (uint32_t)st + 1u;
+                    if (e.t) res_send<1, 2, 5, 6>(k, out, tag, X, Y, XB, YB, cell, a, false, false, inB);
+                    if (e.b) res_send<1, 4, 7, 8>(k, out, tag, X, Y, XB, YB, cell, a, false, false, inB);
+                    if (e.r) res_send<0, 1, 5, 8>(k, out, tag, X, Y, XB, YB, cell, a, e.t, e.b, inB);
+                    if (e.l) res_send<0, 3, 7, 6>(k, out, tag, X, Y, XB, YB, cell, a, e.b, e.t, inB);
+                }
+            }
+            // after the stores: what the neighbours wait for leaves first
+            if constexpr (SAMPLE != kResQuiet) {
+                if (smp) {
+                    if constexpr (SAMPLE == kResExact)
+                        gram_mma_pair(gh, gl, reinterpret_cast<float(&)[8]>(gc));
+                    else
+                        gram_mma(gh, reinterpret_cast<float(&)[8]>(gc));
+                }
+            }
+            x += dx;
+            y += dy;
+            if (x >= bw) {
+                x -= bw;
+                ++y;
+            }
+        }
+        if constexpr (SAMPLE != kResQuiet) {
+            if (smp) {
+                if (warp < nwork)
+                    res_publish(reinterpret_cast<float(&)[8]>(gc), slots + ((nsum & 1) * nw + warp) * kResSlot);
+                ++nsum;
+                pending = true;
+            }
+        }
+        sx = sx + 1 == bw ? 0 : sx + 1;
+        sy = sy + 1 == bh ? 0 : sy + 1;
+        if (!last) __syncthreads();
+    }
+    if constexpr (SAMPLE != kResQuiet) {
+        __syncthreads();
+        if (pending) res_reduce(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
+        __syncthreads();
+        if (nsum)
+            for (int q = c; q < kSums; q += T) atomicAdd(&k.acc[q], res_sum(red, q, par.s));
+    }
+}
+
+// One lattice (a handle): CTA b is block b of gx x gy.
+struct ResidentArgs {
+    ResBlock k;          // x0, y0, bw, bh, ix, iy are the CTA's own
+    float ref[9];        // f^0(rho0, u0)
+    float sinv;          // 1 / s
+    float snref[9];      // -ref / s
+    double s;            // scale of the staged deviations
+};
+
+// The block of column ix and row iy of the grid of blocks.
+__host__ __device__ __forceinline__ void res_place(ResBlock& k, int ix, int iy) {
+    k.ix = ix;
+    k.iy = iy;
+    k.x0 = (int)((long long)ix * k.geo.Lx / k.gx);
+    k.y0 = (int)((long long)iy * k.geo.Ly / k.gy);
+    k.bw = (int)((long long)(ix + 1) * k.geo.Lx / k.gx) - k.x0;
+    k.bh = (int)((long long)(iy + 1) * k.geo.Ly / k.gy) - k.y0;
+}
+
+struct LatticePar {
+    const NoiseKey& key;
+    const CollideConst<float>& cc;
+    const ResidentArgs& a;
+    double s;
+    __device__ __forceinline__ f2 scaled(f2 f, int i) const { return mad(f, f2(a.sinv), f2(a.snref[i])); }
+    __device__ __forceinline__ float ref(int i) const { return a.ref[i]; }
+};
+
+template <int BASIS, int SAMPLE>
+__global__ void __launch_bounds__(kResMaxWarps * 32, 1)
+resident_kernel(const __grid_constant__ ResidentArgs a, const __grid_constant__ CollideConst<float> cc) {
+    extern __shared__ __align__(128) unsigned char res_smem[];
+    ResBlock k = a.k;
+    const int iy = blockIdx.x / k.gx;
+    res_place(k, blockIdx.x - iy * k.gx, iy);
+    resident_run<BASIS, SAMPLE>(k, LatticePar{cc.key, cc, a, a.s}, res_smem);
+}
+
+// Steps of one launch: at least kResMinSteps (fewer cost less one by one).
+constexpr int kResMinSteps = 3;
+constexpr int kResMaxSteps = 1 << 20;
+
+// A lattice's launch: how it is cut, and what the launch needs.
+struct ResidentPlan {
+    int gx = 0, gy = 0;      // 0: no resident launch
+    int threads[2] = {0, 0};
+    size_t smem[2] = {0, 0}; // without, with sampling (0: does not fit)
+    long long mail_words = 0;
+};
+
+// Cut a lattice for the given number of SMs; `cut` = false: one block only.
+ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut);
+// Raise the kernels' dynamic shared memory limit (once per plan).
+cudaError_t resident_prepare(const ResidentPlan& p, int basis);
+cudaError_t resident_step(const ResidentPlan& p, const ResidentArgs& a, const CollideConst<float>& cc, int basis,
+                          bool sample, cudaStream_t s);
+
+}  // namespace flb
