@@ -336,9 +336,11 @@ int flb_batch_destroy(flb_batch b);
  * with times counted from the replica's time 0; clears its sums. */
 int flb_batch_set_sampling(flb_batch b, int32_t slot, int64_t warmup, int64_t every);
 
-/* Enqueue n steps of the batch (one launch each): every live replica below
- * its step limit advances by one time step per launch. With graphs on
- * (flb_batch_set_graph), whole chunks are replayed from a captured CUDA graph.
+/* Enqueue n steps of the batch: every live replica below its step limit
+ * advances by one time step in each. Batches whose replicas fit the SMs' shared
+ * memory (small ones whole, a few larger ones in parts) make calls of three
+ * steps or more in one launch; others take one launch per step, and with graphs
+ * on (flb_batch_set_graph) whole chunks of them from a captured CUDA graph.
  * Errors: FLB_ERR_ARG, FLB_ERR_CUDA. Device errors surface in sync/status. */
 int flb_batch_step(flb_batch b, int64_t n);
 

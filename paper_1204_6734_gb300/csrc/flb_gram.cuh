@@ -125,8 +125,10 @@ __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
 // The same sums from deviations staged as two FP16 numbers, h + l with l the
 // rounding error of h rounded again: 22 bits of a value, so that the products
 // h h + h l + l h carry FP32's accuracy (l l, below 2^-22 of them, is left out).
-// The l block has the layout of the h block, its row 9 zero; the three products
-// share the FP32 accumulators.
+// The l block has the layout of the h block, its row 9 zero. Every 16 nodes
+// start from zero and are added to the sums outside the tensor cores, rounded to
+// nearest: their accumulators cut off instead, which biased the second moments
+// by 1e-6 when they ran over the 24 products of a block of 64 nodes.
 __device__ __forceinline__ void gram_zero_row(__half* blk) {
     reinterpret_cast<uint32_t*>(blk)[9 * (kGramRowHalves / 2) + (threadIdx.x & 31)] = 0u;
 }
@@ -165,12 +167,17 @@ __device__ __forceinline__ void gram_step_pair(uint32_t ld, uint32_t ll, float (
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4+%5];"
                  : "=r"(e0), "=r"(e1), "=r"(e2), "=r"(e3)
                  : "r"(ll), "n"(32 * S));
-    mma16816(c, 0, d0, d1, d2, d3, d0, d2);
-    mma16816(c, 4, d0, d1, d2, d3, d1, d3);
-    mma16816(c, 0, d0, d1, d2, d3, e0, e2);
-    mma16816(c, 4, d0, d1, d2, d3, e1, e3);
-    mma16816(c, 0, e0, e1, e2, e3, d0, d2);
-    mma16816(c, 4, e0, e1, e2, e3, d1, d3);
+    float p[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) p[q] = 0.f;
+    mma16816(p, 0, d0, d1, d2, d3, d0, d2);
+    mma16816(p, 4, d0, d1, d2, d3, d1, d3);
+    mma16816(p, 0, d0, d1, d2, d3, e0, e2);
+    mma16816(p, 4, d0, d1, d2, d3, e1, e3);
+    mma16816(p, 0, e0, e1, e2, e3, d0, d2);
+    mma16816(p, 4, e0, e1, e2, e3, d1, d3);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) c[q] += p[q];
 }
 
 __device__ __forceinline__ void gram_mma_pair(const GramLane& g, const GramLane& l, float (&c)[8]) {

@@ -16,8 +16,6 @@ const void* kernel_of(int basis, bool sample) {
     return sample ? (const void*)resident_kernel<2, kResStaged> : (const void*)resident_kernel<2, kResQuiet>;
 }
 
-constexpr size_t kSmemMax = 227 * 1024;
-
 // Estimated microseconds of a step (f-norm, no sampling): wp warp passes of 64
 // nodes on the four schedulers of an SM; blocks that exchange add their words'
 // trip through L2 and the passes whose lanes move them (a row on the edge; all
@@ -27,12 +25,16 @@ constexpr size_t kSmemMax = 227 * 1024;
 // 130 blocks 5.2 / 3.7 / 3.5 / 4.1; 512 x 512 in 128 x 1 7.0, 2 x 74 7.1, 8 x 19
 // 7.9; 4000 x 20 in 1 / 2 / 4 / 7 x 20 20.0 / 10.5 / 5.7 / 4.9; 1000 x 750 in
 // 150 x 1 16.4, 2 x 75 22.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
-double step_us(int wp, int gx, int gy, int bw, int bh) {
+}  // namespace
+
+double resident_step_us(int wp, int gx, int gy, int bw, int bh) {
     double t = std::max(1.75, 0.69 * ((wp + 3) / 4) + 0.3);
     if (gy > 1) t += 0.3 + 0.072 * bw / 32.0 + (bh == 1 ? 1.2 : 0.0);   // one row: two waits in a row
     if (gx > 1) t += 1.0 + 0.08 * std::min(wp, bh);
     return t;
 }
+
+namespace {
 
 // The same for one launch per step, from the measured 6.2 (up to 300 x 130),
 // 8.2 (400 x 300), 10.3 (512 x 512), 19.8 (1000 x 750), 20.8 (900 x 900);
@@ -56,8 +58,8 @@ ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
             const int swarps = std::min(kResMaxWarps, wp + 3);
             const size_t q = res_smem_bytes((int)cells, kResQuiet, warps);
             const size_t t = res_smem_bytes((int)cells, kResStaged, swarps);
-            if (q > kSmemMax) continue;
-            const double c = step_us(wp, gx, gy, bw, bh);
+            if (q > kResSmemMax) continue;
+            const double c = resident_step_us(wp, gx, gy, bw, bh);
             if (c >= cost) continue;
             cost = c;
             best.gx = gx;
@@ -65,7 +67,7 @@ ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
             best.threads[0] = warps * 32;
             best.threads[1] = swarps * 32;
             best.smem[0] = q;
-            best.smem[1] = t <= kSmemMax ? t : 0;
+            best.smem[1] = t <= kResSmemMax ? t : 0;
             best.mail_words = res_mail_words(Lx, Ly, gx, gy);
         }
     }
@@ -77,7 +79,7 @@ cudaError_t resident_prepare(const ResidentPlan& p, int basis) {
     cudaError_t ce = cudaSuccess;
     for (int smp = 0; smp < 2 && ce == cudaSuccess; ++smp)
         if (p.smem[smp])
-            ce = cudaFuncSetAttribute(kernel_of(basis, smp), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+            ce = cudaFuncSetAttribute(kernel_of(basis, smp), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
     return ce;
 }
 

@@ -520,6 +520,11 @@ struct ResidentPlan {
     long long mail_words = 0;
 };
 
+constexpr size_t kResSmemMax = 227 * 1024;
+
+// Estimated microseconds of a step of a block of bw x bh nodes, wp warp passes,
+// of a lattice cut into gx x gy blocks.
+double resident_step_us(int wp, int gx, int gy, int bw, int bh);
 // Cut a lattice for the given number of SMs; `cut` = false: one block only.
 ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut);
 // Raise the kernels' dynamic shared memory limit (once per plan).
