@@ -15,6 +15,7 @@
 #include "flb_runtime.h"
 #include "flb_internal.h"
 #include "flb_io.cuh"
+#include "flb_step64.cuh"
 #include "flb_structure.h"
 #include "flb_kernels.cuh"
 #include "flb_resident.cuh"
@@ -189,14 +190,21 @@ state_difference_kernel(StateView a, StateView b, double* partials) {
 template <class T>
 __global__ void noise_draws_kernel(uint64_t seed, uint32_t replica, uint32_t step,
                                    const uint32_t* nodes, int n, uint32_t* fields,
-                                   double* normals) {
+                                   double* normals, NoiseTables tab) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const NoiseKey key = make_noise_key(seed, replica);   // per-thread copy, test hook only
     uint32_t f[6];
     node_fields(key, nodes[k], step, f);
     T z[6];
-    box_muller(f, z);
+    if constexpr (sizeof(T) == 8) {   // as the FP64 step: by table where there is one
+        if (tab.radius)
+            TableNoise{key, nodes[k], step, tab}(z);
+        else
+            box_muller(f, z);
+    } else {
+        box_muller(f, z);
+    }
     for (int q = 0; q < 6; ++q) {
         fields[k * 6 + q] = f[q];
         normals[k * 6 + q] = (double)z[q];
@@ -276,7 +284,11 @@ struct flb_lattice_s {
     void* buf[2];
     int cur;             // buf[cur] holds f*(t-1), the source of the next pull
     double* partials;
-    int nblocks;         // grid of the step kernel
+    int nblocks;         // grid of the generic step kernel and the reductions
+    int blocks64 = 0;    // grid of the FP64 step
+    int sms = 1;
+    double* pending64 = nullptr;   // partial sums of the last FP64 step, not yet in acc
+    NoiseTables noise;   // FP64 lattices
     double* acc;         // kSums running sums
     double* small;       // basis (81) + finalize output (171) + conservation (3)
     DevError* err;
@@ -329,7 +341,7 @@ int step_grid(const Geometry& g, int sms) {
 
 struct Layout {
     size_t buf_bytes, partial_off, acc_off, small_off, err_off, total;
-    int nblocks, npartials;
+    int nblocks, npartials, blocks64;
 };
 
 Layout layout(const flb_params* p, int sms) {
@@ -338,7 +350,8 @@ Layout layout(const flb_params* p, int sms) {
     L.nblocks = step_grid(g, sms);
     L.buf_bytes = align_up((size_t)(9 * g.plane) * elem_size(p->precision));
     size_t off = 2 * L.buf_bytes;
-    L.npartials = L.nblocks;
+    L.blocks64 = p->precision == FLB_FP64 ? step64_blocks((long long)p->Lx * p->Ly, sms) : 0;
+    L.npartials = std::max(L.nblocks, 2 * L.blocks64);   // FP64: of two steps in turn
     L.partial_off = off;
     off += align_up(sizeof(double) * (size_t)L.npartials * kSums);
     L.acc_off = off;
@@ -354,30 +367,56 @@ Layout layout(const flb_params* p, int sms) {
 int cuda_rc(cudaError_t e) { return e == cudaSuccess ? FLB_OK : FLB_ERR_CUDA; }
 
 
-template <class T, int BASIS, bool SAMPLE>
-cudaError_t launch_step_t(flb_lattice h) {
-    StepArgs<T> a;
-    a.src = (const T*)h->buf[h->cur];
-    a.dst = (T*)h->buf[h->cur ^ 1];
+// The generic FP32 kernel (one node per thread, plain loads).
+template <int BASIS, bool SAMPLE>
+cudaError_t launch_generic_t(flb_lattice h) {
+    StepArgs<float> a;
+    a.src = (const float*)h->buf[h->cur];
+    a.dst = (float*)h->buf[h->cur ^ 1];
     a.geo = h->geo;
     a.step = (uint32_t)h->t;
     a.node0 = h->node0;
     a.partials = h->partials;
     a.err = h->err;
-    a.lut = (const T*)(sizeof(T) == 8 ? (const void*)h->lut64 : (const void*)h->lut32);
-    for (int i = 0; i < 9; ++i) a.ref[i] = (T)h->ref[i];
-    step_kernel<T, BASIS, SAMPLE><<<h->nblocks, kStepThreads, 0, h->stream>>>(
-        a, collide_const<T>(&h->p));
+    a.lut = h->lut32;
+    for (int i = 0; i < 9; ++i) a.ref[i] = (float)h->ref[i];
+    step_kernel<float, BASIS, SAMPLE><<<h->nblocks, kStepThreads, 0, h->stream>>>(a, collide_const<float>(&h->p));
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t launch_step_p(flb_lattice h, bool sample) {
-    if (h->p.basis == FLB_BASIS_STANDARD)
-        return sample ? launch_step_t<T, 0, true>(h) : launch_step_t<T, 0, false>(h);
-    if (h->p.basis == FLB_BASIS_LOCAL)
-        return sample ? launch_step_t<T, 1, true>(h) : launch_step_t<T, 1, false>(h);
-    return sample ? launch_step_t<T, 2, true>(h) : launch_step_t<T, 2, false>(h);
+cudaError_t launch_generic(flb_lattice h, bool sample) {
+    if (h->p.basis == FLB_BASIS_STANDARD) return sample ? launch_generic_t<0, true>(h) : launch_generic_t<0, false>(h);
+    if (h->p.basis == FLB_BASIS_LOCAL) return sample ? launch_generic_t<1, true>(h) : launch_generic_t<1, false>(h);
+    return sample ? launch_generic_t<2, true>(h) : launch_generic_t<2, false>(h);
+}
+
+// FP64: leaves the step's partial sums pending; the next sampled step, or
+// flush64 at the end of the call, adds them to h->acc.
+cudaError_t launch_step64(flb_lattice h, bool sample) {
+    Step64Args a;
+    a.src = (const double*)h->buf[h->cur];
+    a.dst = (double*)h->buf[h->cur ^ 1];
+    a.geo = h->geo;
+    a.step = (uint32_t)h->t;
+    a.node0 = h->node0;
+    a.blocks = h->blocks64;
+    a.partials = h->pending64 == h->partials ? h->partials + (size_t)h->blocks64 * kSums : h->partials;
+    a.prev = h->pending64;
+    a.acc = h->acc;
+    a.err = h->err;
+    a.lut = h->lut64;
+    a.noise = h->noise;
+    for (int i = 0; i < 9; ++i) a.ref[i] = h->ref[i];
+    const cudaError_t ce = step64(a, collide_const<double>(&h->p), h->p.basis, sample, h->sms, h->stream);
+    if (sample && ce == cudaSuccess) h->pending64 = a.partials;
+    return ce;
+}
+
+cudaError_t flush64(flb_lattice h) {
+    if (!h->pending64) return cudaSuccess;
+    const cudaError_t ce = step64_flush(h->pending64, h->blocks64, h->acc, h->stream);
+    h->pending64 = nullptr;
+    return ce;
 }
 
 // Pipelined FP32 kernel: also reduces the sampled sums into h->acc itself.
@@ -468,8 +507,8 @@ bool uses_tma(flb_lattice h) {
     return h->p.precision == FLB_FP32 && h->variant != FLB_KERNEL_GENERIC;
 }
 
-// The pipelined kernels (FP32, FP16 store) add their sums to h->acc themselves.
-bool reduces_in_kernel(flb_lattice h) { return uses_tma(h) || h->p.precision == FLB_FP16_DEV; }
+// Every step but the generic kernel's adds its sums to h->acc itself.
+bool reduces_in_kernel(flb_lattice h) { return uses_tma(h) || h->p.precision != FLB_FP32; }
 
 DevCodec dev_codec(flb_lattice h) {
     DevCodec c;
@@ -502,10 +541,10 @@ cudaError_t launch_step_fp16(flb_lattice h, bool sample) {
 // fields: where the pipelined FP32 kernel writes the structure-factor fields
 // of this step's pre-collision state (nullptr: not sampled by the step).
 cudaError_t launch_step(flb_lattice h, bool sample, float* fields = nullptr) {
-    if (h->p.precision == FLB_FP64) return launch_step_p<double>(h, sample);
+    if (h->p.precision == FLB_FP64) return launch_step64(h, sample);
     if (h->p.precision == FLB_FP16_DEV) return launch_step_fp16(h, sample);
     if (uses_tma(h)) return launch_step_tma(h, sample, fields);
-    return launch_step_p<float>(h, sample);
+    return launch_generic(h, sample);
 }
 
 int check_device_error(flb_lattice h) {
@@ -580,6 +619,8 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
     h->small = (double*)(h->ws + L.small_off);
     h->err = (DevError*)(h->ws + L.err_off);
     h->nblocks = L.nblocks;
+    h->blocks64 = L.blocks64;
+    h->sms = sms;
     h->variant = FLB_KERNEL_AUTO;
     h->cur = 0;
     feq_host(p->rho0, p->ux0, p->uy0, h->ref);
@@ -614,6 +655,7 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
         lut_tables(&h->lut32, &h->lut64) != FLB_OK)
         ce = cudaErrorUnknown;
     h->tma_quiet.ready = false;
+    if (ce == cudaSuccess && p->precision == FLB_FP64) h->noise = noise_tables();
     if (ce == cudaSuccess && p->precision == FLB_FP32) {
         ce = tma_plan(&h->tma, h->buf[0], h->buf[1], h->geo, tensor ? tensor_nw : 0);
         // steps without sampling: 16 colliding warps in the f-norm bases
@@ -847,11 +889,15 @@ int flb_step(flb_lattice h, int64_t n) {
             ce = cudaGetLastError();
         }
         if (sample) h->nsamp += N;
-        if (ce != cudaSuccess) return FLB_ERR_CUDA;
+        if (ce != cudaSuccess) {
+            flush64(h);
+            return FLB_ERR_CUDA;
+        }
         h->t += 1;
         h->cur ^= 1;
         ++s;
     }
+    if (flush64(h) != cudaSuccess) return FLB_ERR_CUDA;
     return FLB_OK;
 }
 
@@ -1184,10 +1230,10 @@ int flb_noise_draws(uint64_t seed, uint32_t replica, uint32_t step, const uint32
         const int grid = (n + 127) / 128;
         if (precision == FLB_FP64)
             noise_draws_kernel<double><<<grid, 128>>>(seed, replica, step, d_nodes, n, d_fields,
-                                                      d_normals);
+                                                      d_normals, noise_tables());
         else
             noise_draws_kernel<float><<<grid, 128>>>(seed, replica, step, d_nodes, n, d_fields,
-                                                     d_normals);
+                                                     d_normals, NoiseTables());
         ce = cudaGetLastError();
     }
     if (ce == cudaSuccess)

@@ -1,7 +1,7 @@
 // flb_vec.cuh -- arithmetic types of the collision.
 //
 // The collision is written once, over a "lane type" V:
-//   double  -- FP64 (parity mode), IEEE division and square roots;
+//   double  -- FP64 (parity mode), IEEE division and square roots, rsqrt;
 //   float   -- FP32, SFU reciprocal / square roots;
 //   f2      -- two FP32 nodes per thread in Blackwell's packed FP32x2
 //              instructions (add/sub/mul/fma .f32x2, sm_100+): one issue slot
@@ -21,7 +21,7 @@ __device__ __forceinline__ double mad(double a, double b, double c) { return fma
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 
 __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }   // within 1 ulp, a third of 1.0 / sqrt(x)
 __device__ __forceinline__ double sqr(double x) { return sqrt(x); }
 
 __device__ __forceinline__ float rcp(float x) {
