@@ -87,6 +87,12 @@ __device__ __forceinline__ void gram_store(uint32_t st, f2 h) {
                  "r"(*reinterpret_cast<const uint32_t*>(&v)));
 }
 
+template <int I>
+__device__ __forceinline__ void gram_store_raw(uint32_t st, __half2 v) {
+    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(st), "n"(2 * kGramRowHalves * I),
+                 "r"(*reinterpret_cast<const uint32_t*>(&v)));
+}
+
 template <int S>
 __device__ __forceinline__ void gram_step(uint32_t ld, float (&c)[8]) {
     uint32_t d0, d1, d2, d3;
@@ -113,6 +119,20 @@ __device__ __forceinline__ void gram_stage(const GramLane& g, const f2 (&h)[9]) 
     gram_store<8>(g.st, h[8]);
 }
 
+// The same from values that are FP16 already.
+__device__ __forceinline__ void gram_stage_raw(const GramLane& g, const __half2 (&h)[9]) {
+    __syncwarp();
+    gram_store_raw<0>(g.st, h[0]);
+    gram_store_raw<1>(g.st, h[1]);
+    gram_store_raw<2>(g.st, h[2]);
+    gram_store_raw<3>(g.st, h[3]);
+    gram_store_raw<4>(g.st, h[4]);
+    gram_store_raw<5>(g.st, h[5]);
+    gram_store_raw<6>(g.st, h[6]);
+    gram_store_raw<7>(g.st, h[7]);
+    gram_store_raw<8>(g.st, h[8]);
+}
+
 // Add the staged block to c: four 16-node steps of two mma.m16n8k16 each.
 __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
     __syncwarp();
@@ -120,6 +140,18 @@ __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
     gram_step<1>(g.ld, c);
     gram_step<2>(g.ld, c);
     gram_step<3>(g.ld, c);
+}
+
+// As gram_mma, with the block's sums started from zero and added to c outside the
+// tensor cores, rounded to nearest (their accumulators cut off): for values that
+// are FP16 numbers to begin with, whose products FP32 holds exactly.
+__device__ __forceinline__ void gram_mma_rn(const GramLane& g, float (&c)[8]) {
+    float p[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) p[q] = 0.f;
+    gram_mma(g, p);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) c[q] += p[q];
 }
 
 // The same sums from deviations staged as two FP16 numbers, h + l with l the
