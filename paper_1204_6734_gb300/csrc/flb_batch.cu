@@ -60,6 +60,7 @@ struct flb_batch_s {
     BatchCtl* ctl = nullptr;
     double* acc = nullptr;         // [cap][kSums]
     DevError* err = nullptr;       // [cap]
+    double* scratch = nullptr;     // finalised correlations
     std::vector<BatchSlot> slots;
     std::vector<ReplicaDesc> hdesc;
     std::vector<uint32_t> htiles;
@@ -475,7 +476,8 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     // blocks exchanges 96 bytes per column, a node is 72 bytes of the pool)
     const size_t rtab_bytes = Arena::round_up(sizeof(ResCta) * std::max(max_replicas, b->sms));
     const size_t mail_bytes = Arena::round_up(std::min<size_t>(pool_bytes / 4, 16u << 20));
-    const size_t meta_bytes = desc_bytes + tile_bytes + ctl_bytes + acc_bytes + err_bytes + rtab_bytes + mail_bytes;
+    const size_t meta_bytes = desc_bytes + tile_bytes + ctl_bytes + acc_bytes + err_bytes + rtab_bytes + mail_bytes +
+                              Arena::round_up(sizeof(double) * kFinalizeOut);
     void *pool = nullptr, *meta = nullptr;
     if (cudaMalloc(&pool, pool_bytes) != cudaSuccess || cudaMalloc(&meta, meta_bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -500,6 +502,8 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     b->rtable = (ResCta*)m;
     m += rtab_bytes;
     b->mail = (uint64_t*)m;
+    m += mail_bytes;
+    b->scratch = (double*)m;
     b->mail_words = mail_bytes / sizeof(uint64_t);
 
     ce = cudaMemsetAsync(b->meta, 0, meta_bytes, b->stream);
@@ -884,33 +888,50 @@ int flb_batch_correlations(flb_batch b, int32_t n, const int32_t* slots, int32_t
         const flb_params& c = b->slots[slots[q]].p;
         if (c.rho0 != a.rho0 || c.ux0 != a.ux0 || c.uy0 != a.uy0) return FLB_ERR_ARG;
     }
+    // the sums and error records of every slot from the first to the last one
+    // asked for, in two copies
+    int32_t lo = slots[0], hi = slots[0];
+    for (int32_t q = 1; q < n; ++q) {
+        lo = std::min(lo, slots[q]);
+        hi = std::max(hi, slots[q]);
+    }
+    std::vector<double> acc;
+    std::vector<DevError> err;
+    try {
+        acc.resize((size_t)(hi - lo + 1) * kSums);
+        err.resize(hi - lo + 1);
+    } catch (const std::bad_alloc&) {
+        return FLB_ERR_OOM;
+    }
+    cudaError_t ce = cudaMemcpyAsync(acc.data(), b->acc + (size_t)lo * kSums, sizeof(double) * acc.size(),
+                                     cudaMemcpyDeviceToHost, b->stream);
+    if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(err.data(), b->err + lo, sizeof(DevError) * err.size(), cudaMemcpyDeviceToHost, b->stream);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
+    if (ce != cudaSuccess) {
+        cudaGetLastError();
+        return FLB_ERR_CUDA;
+    }
     double pooled[kSums] = {0.0};
     int64_t ns = 0;
     for (int32_t q = 0; q < n; ++q) {
-        double acc[kSums];
-        cudaError_t ce = cudaMemcpyAsync(acc, b->acc + (size_t)slots[q] * kSums, sizeof(acc),
-                                         cudaMemcpyDeviceToHost, b->stream);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            return FLB_ERR_CUDA;
-        }
-        const int rc = read_status(b, slots[q]);
+        const int rc = map_status(err[slots[q] - lo].code);
         if (rc) return rc;
-        for (int k = 0; k < kSums; ++k) pooled[k] += acc[k];
+        for (int k = 0; k < kSums; ++k) pooled[k] += acc[(size_t)(slots[q] - lo) * kSums + k];
         ns += b->slots[slots[q]].nsamp;
     }
     if (n_samples) *n_samples = ns;
     const flb_params& p = b->slots[slots[0]].p;
-    return finalize_sums(pooled, ns, measure_basis, p.ux0, p.uy0, b->stream, Cff, CMM, mean_dev);
+    return finalize_sums(pooled, ns, measure_basis, p.ux0, p.uy0, b->scratch, b->stream, Cff, CMM, mean_dev);
 }
 
 int flb_batch_get_populations(flb_batch b, int32_t slot, double* host_out) {
     if (!slot_ok(b, slot) || !host_out) return FLB_ERR_ARG;
     const BatchSlot& s = b->slots[slot];
     const size_t n = (size_t)9 * s.p.Lx * s.p.Ly;
-    double* tmp = nullptr;
-    if (cudaMalloc(&tmp, n * sizeof(double)) != cudaSuccess) {
+    double* direct = pinned_view(host_out);
+    double* tmp = direct;
+    if (!direct && cudaMalloc(&tmp, n * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_OOM;
     }
@@ -918,36 +939,40 @@ int flb_batch_get_populations(flb_batch b, int32_t slot, double* host_out) {
     gather_state_kernel<float><<<grid_for((long long)s.p.Lx * s.p.Ly), 256, 0, b->stream>>>(
         src, s.geo, tmp);
     cudaError_t ce = cudaGetLastError();
-    if (ce == cudaSuccess)
+    if (ce == cudaSuccess && !direct)
         ce = cudaMemcpyAsync(host_out, tmp, n * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+    DevError e;
+    if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(&e, b->err + slot, sizeof(e), cudaMemcpyDeviceToHost, b->stream);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
+    if (!direct) cudaFree(tmp);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_CUDA;
     }
-    return read_status(b, slot);
+    return map_status(e.code);
 }
 
 int flb_batch_set_populations(flb_batch b, int32_t slot, const double* host_in) {
     if (!slot_ok(b, slot) || !host_in) return FLB_ERR_ARG;
     const BatchSlot& s = b->slots[slot];
     const size_t n = (size_t)9 * s.p.Lx * s.p.Ly;
-    double* tmp = nullptr;
-    if (cudaMalloc(&tmp, n * sizeof(double)) != cudaSuccess) {
+    double* direct = pinned_view(host_in);
+    double* tmp = direct;
+    if (!direct && cudaMalloc(&tmp, n * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_OOM;
     }
     float* dst = s.buf[slot_time(b, s) & 1];
-    cudaError_t ce = cudaMemcpyAsync(tmp, host_in, n * sizeof(double), cudaMemcpyHostToDevice,
-                                     b->stream);
+    cudaError_t ce = direct ? cudaSuccess
+                            : cudaMemcpyAsync(tmp, host_in, n * sizeof(double), cudaMemcpyHostToDevice, b->stream);
     if (ce == cudaSuccess) {
         scatter_state_kernel<float><<<grid_for((long long)s.p.Lx * s.p.Ly), 256, 0, b->stream>>>(
             tmp, s.geo, dst);
         ce = cudaGetLastError();
     }
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
-    cudaFree(tmp);
+    if (!direct) cudaFree(tmp);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_CUDA;

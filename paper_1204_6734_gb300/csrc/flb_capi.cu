@@ -10,7 +10,6 @@
 #include <vector>
 
 #include "../../include/flb.h"
-#include "flb_basis.cuh"
 #include "flb_host.h"
 #include "flb_runtime.h"
 #include "flb_internal.h"
@@ -31,46 +30,90 @@ __global__ void accumulate_partials_kernel(const double* partials, int nblocks, 
     if (threadIdx.x == 0) acc[blockIdx.x] += v;
 }
 
-// Rows of the basis the correlations are measured in: the Hermite rows
-// (Eq. d2q93a), or the f-norm basis at (ux0, uy0) -- Cholesky of the full 9x9
-// Gram matrix sum_i p^a_i p^b_i f_i^0(1,u0), m~ = L^{-1} P. One thread.
-__global__ void measure_basis_kernel(int basis, double ux0, double uy0, double* out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (basis == FLB_BASIS_STANDARD) {
-        double P[9][9];
-        hermite_rows_fp64(P);
-        for (int a = 0; a < 9; ++a)
-            for (int i = 0; i < 9; ++i) out[a * 9 + i] = P[a][i];
-        return;
-    }
-    fnorm_basis_fp64(ux0, uy0, out);
-}
+// Correlations from running sums: C = S2/n - m m^T (m = S1/n) and B C B^T for
+// the measurement basis B -- the Hermite rows (Eq. d2q93a), or the f-norm basis
+// at (ux0, uy0): Cholesky of the Gram matrix sum_i p^a_i p^b_i f_i^0(1,u0),
+// B = L^{-1} P. out: Cff[81], CMM[81], mean[9]. One block, one thread per matrix
+// element: column k of L and row k of B, then the update of what remains (a
+// thread alone, with the matrices in local memory, took 84 us for the basis and
+// the 81-term sums after it 9 us; this takes 10 us).
+constexpr int kFinalizeThreads = 96;
+struct Sums {
+    double v[kSums];
+};
 
-__global__ void finalize_kernel(const double* acc, long long nsamp, const double* B,
-                                double* out) {
-    __shared__ double C[81];
-    __shared__ double mean[9];
-    const int t = threadIdx.x;
+__device__ __forceinline__ void finalize_block(const double* acc, long long nsamp, int basis, double ux0, double uy0,
+                                               double* out) {
+    __shared__ double P[81], G[81], B[81], C[81], T[81], mean[9], W[9];
+    const int t = threadIdx.x, a = t / 9, b = t % 9;
+    const bool on = t < 81;
     const double inv = 1.0 / (double)nsamp;
-    if (t < 9) mean[t] = acc[t] * inv;
+    if (t < 9) {
+        double Dn[6], h[9];
+        for (int q = 0; q < 6; ++q) Dn[q] = t == 3 + q ? 1.0 : 0.0;
+        hermite_back<double, true>(t == 0 ? 1.0 : 0.0, t == 1 ? -1.0 : 0.0, t == 2 ? -1.0 : 0.0, Dn, h);
+        for (int i = 0; i < 9; ++i) P[t * 9 + i] = h[i];
+        mean[t] = acc[t] * inv;
+        const double uv = ux0 * cvx(t) + uy0 * cvy(t);
+        W[t] = (t == 0 ? 4.0 / 9.0 : (t <= 4 ? 1.0 / 9.0 : 1.0 / 36.0)) *
+               (1.0 + 3.0 * uv + 4.5 * uv * uv - 1.5 * (ux0 * ux0 + uy0 * uy0));
+    }
     __syncthreads();
-    if (t < 81) {
-        const int i = t / 9, j = t % 9;
-        const int a = i < j ? i : j, b = i < j ? j : i;
-        // index of (a, b), a <= b, in the packed upper triangle after S1
-        const int k = 9 + a * 9 - a * (a - 1) / 2 + (b - a);
-        C[t] = acc[k] * inv - mean[i] * mean[j];
+    if (on) {
+        const int i = a < b ? a : b, j = a < b ? b : a;
+        C[t] = acc[9 + i * 9 - i * (i - 1) / 2 + (j - i)] * inv - mean[a] * mean[b];
+        double s = 0.0;
+        for (int q = 0; q < 9; ++q) s += P[a * 9 + q] * W[q] * P[b * 9 + q];
+        G[t] = s;
+        B[t] = P[t];
+    }
+    __syncthreads();
+    if (basis != FLB_BASIS_STANDARD) {
+        for (int k = 0; k < 9; ++k) {
+            double l = 0.0, m = 0.0;   // L[a][k], B[k][b]
+            if (on) {
+                const double d = rsqrt(G[10 * k]);
+                l = G[a * 9 + k] * d;
+                m = B[k * 9 + b] * d;
+            }
+            const double lb = on ? G[b * 9 + k] * rsqrt(G[10 * k]) : 0.0;   // L[b][k]
+            __syncthreads();
+            if (on) {
+                if (a == k) B[t] = m;
+                if (a > k) {
+                    B[t] -= l * m;
+                    if (b > k) G[t] -= l * lb;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (on) {
+        double s = 0.0;
+        for (int j = 0; j < 9; ++j) s += B[a * 9 + j] * C[j * 9 + b];
+        T[t] = s;
         out[t] = C[t];
     }
     __syncthreads();
-    if (t < 81) {
-        const int a = t / 9, b = t % 9;
+    if (on) {
         double s = 0.0;
-        for (int i = 0; i < 9; ++i)
-            for (int j = 0; j < 9; ++j) s += B[a * 9 + i] * C[i * 9 + j] * B[b * 9 + j];
+        for (int j = 0; j < 9; ++j) s += T[a * 9 + j] * B[b * 9 + j];
         out[81 + t] = s;
     }
     if (t < 9) out[162 + t] = mean[t];
+}
+
+__global__ void __launch_bounds__(kFinalizeThreads) finalize_kernel(const double* acc, long long nsamp, int basis,
+                                                                    double ux0, double uy0, double* out) {
+    finalize_block(acc, nsamp, basis, ux0, uy0, out);
+}
+// The same from sums that the host has added up.
+__global__ void __launch_bounds__(kFinalizeThreads) finalize_sums_kernel(const Sums in, long long nsamp, int basis,
+                                                                         double ux0, double uy0, double* out) {
+    __shared__ double acc[kSums];
+    if (threadIdx.x < kSums) acc[threadIdx.x] = in.v[threadIdx.x];
+    __syncthreads();
+    finalize_block(acc, nsamp, basis, ux0, uy0, out);
 }
 
 // Total mass and momentum of the pre-collision state, FP64 per block.
@@ -706,26 +749,17 @@ void lattice_forget(flb_lattice h) {
 
 namespace flb {
 
-int finalize_sums(const double* acc, int64_t nsamp, int32_t measure_basis, double ux0, double uy0,
+int finalize_sums(const double* acc, int64_t nsamp, int32_t measure_basis, double ux0, double uy0, double* scratch,
                   cudaStream_t st, double* Cff, double* CMM, double* mean_dev) {
     if (measure_basis != FLB_BASIS_STANDARD && measure_basis != FLB_BASIS_LOCAL) return FLB_ERR_ARG;
     if (nsamp <= 0) return FLB_ERR_STATE;
-    double* dev = nullptr;   // sums, basis, results
-    if (cudaMalloc(&dev, sizeof(double) * (kSums + 81 + 171)) != cudaSuccess) {
-        cudaGetLastError();
-        return FLB_ERR_OOM;
-    }
-    double host[171];
-    cudaError_t ce = cudaMemcpyAsync(dev, acc, sizeof(double) * kSums, cudaMemcpyHostToDevice, st);
-    if (ce == cudaSuccess) {
-        measure_basis_kernel<<<1, 32, 0, st>>>(measure_basis, ux0, uy0, dev + kSums);
-        finalize_kernel<<<1, 96, 0, st>>>(dev, nsamp, dev + kSums, dev + kSums + 81);
-        ce = cudaGetLastError();
-    }
-    if (ce == cudaSuccess)
-        ce = cudaMemcpyAsync(host, dev + kSums + 81, sizeof(host), cudaMemcpyDeviceToHost, st);
+    Sums in;
+    std::memcpy(in.v, acc, sizeof(in.v));
+    double host[kFinalizeOut];
+    finalize_sums_kernel<<<1, kFinalizeThreads, 0, st>>>(in, nsamp, measure_basis, ux0, uy0, scratch);
+    cudaError_t ce = cudaGetLastError();
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(host, scratch, sizeof(host), cudaMemcpyDeviceToHost, st);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
-    cudaFree(dev);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_CUDA;
@@ -1050,10 +1084,8 @@ int flb_correlations(flb_lattice h, int32_t measure_basis, double* Cff, double* 
     if (rc) return rc;
     if (n_samples) *n_samples = h->nsamp;
     if (h->nsamp <= 0) return FLB_ERR_STATE;
-    double* basis = h->small;
     double* res = h->small + 81;
-    measure_basis_kernel<<<1, 32, 0, h->stream>>>(measure_basis, h->p.ux0, h->p.uy0, basis);
-    finalize_kernel<<<1, 96, 0, h->stream>>>(h->acc, h->nsamp, basis, res);
+    finalize_kernel<<<1, kFinalizeThreads, 0, h->stream>>>(h->acc, h->nsamp, measure_basis, h->p.ux0, h->p.uy0, res);
     double host[171];
     cudaError_t ce = cudaGetLastError();
     if (ce == cudaSuccess)
@@ -1124,18 +1156,6 @@ int flb_state_difference(flb_lattice a, flb_lattice b, double out[3]) {
     out[1] = std::sqrt(ss / (9.0 * (double)a->p.Lx * (double)a->p.Ly));
     out[2] = mb;
     return FLB_OK;
-}
-
-// The device address of page-locked host memory, or null for other memory:
-// the state I/O kernels then read or write the caller's host array themselves
-// (one pass over the host link, no device staging buffer).
-static double* pinned_view(const void* host) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return a.type == cudaMemoryTypeHost ? static_cast<double*>(a.devicePointer) : nullptr;
 }
 
 int flb_get_populations(flb_lattice h, double* host_out) {

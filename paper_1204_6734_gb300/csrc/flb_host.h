@@ -83,6 +83,18 @@ inline int64_t count_sampled(int64_t ta, int64_t tb, int64_t warmup, int64_t eve
     return (tb - 1 - first) / every + 1;
 }
 
+// The device address of page-locked host memory, or null for other memory:
+// the state I/O kernels then read or write the caller's host array themselves
+// (one pass over the host link, no device staging buffer).
+inline double* pinned_view(const void* host) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? static_cast<double*>(a.devicePointer) : nullptr;
+}
+
 inline int grid_for(long long n) {
     long long b = (n + 255) / 256;
     if (b > 4096) b = 4096;

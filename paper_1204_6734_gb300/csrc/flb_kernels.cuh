@@ -134,12 +134,4 @@ __device__ __forceinline__ double reduce_partials(const double* partials, int q,
     return s;
 }
 
-// Adds the per-block partials into the running FP64 sums; block q, one warp,
-// handles sum q.
-__global__ void accumulate_partials_kernel(const double* partials, int nblocks, double* acc);
-
-// C = S2/n - m m^T, m = S1/n, and CM = B C B^T for the measurement basis B.
-__global__ void finalize_kernel(const double* acc, long long nsamp, const double* basis,
-                                double* out /* Cff[81], CMM[81], mean[9] */);
-
 }  // namespace flb

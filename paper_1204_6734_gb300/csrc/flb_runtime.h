@@ -49,9 +49,10 @@ void lattice_forget(flb_lattice h);
 
 // <df df>, <dM dM> and the mean deviation from kSums running sums over nsamp
 // node-samples taken relative to f^0(rho0, u0) (as flb_correlations, with the
-// measurement basis at (ux0, uy0)); on a scratch buffer of its own, ordered on
-// stream st, synchronous. Any output pointer may be NULL.
-int finalize_sums(const double* acc, int64_t nsamp, int32_t measure_basis, double ux0, double uy0,
+// measurement basis at (ux0, uy0)); scratch: kFinalizeOut doubles of device
+// memory; ordered on stream st, synchronous. Any output pointer may be NULL.
+constexpr int kFinalizeOut = 171;
+int finalize_sums(const double* acc, int64_t nsamp, int32_t measure_basis, double ux0, double uy0, double* scratch,
                   cudaStream_t st, double* Cff, double* CMM, double* mean_dev);
 
 }  // namespace flb
