@@ -149,8 +149,7 @@ cudaError_t launch(flb_batch_s* b, bool sample, cudaStream_t s) {
     void* params[1] = {(void*)&a};
     const BatchVariant& v = kBatchVariants[b->tile];
     const int warps = v.nw + (sample && !v.tensor() ? kSamplers : 1);
-    return cudaLaunchKernel(kernel_for(b, sample), dim3(b->grid), dim3(warps * 32), params,
-                            batch_smem_bytes(b->tile), s);
+    return launch_dependent(kernel_for(b, sample), dim3(b->grid), dim3(warps * 32), params, batch_smem_bytes(b->tile), s);
 }
 
 void drop_graphs(flb_batch_s* b) {

@@ -255,8 +255,7 @@ batch_step_kernel(const BatchArgs a) {
     __half* gram = reinterpret_cast<__half*>(cur_s + NW);
 
     const int warp = threadIdx.x >> 5, lane_id = threadIdx.x & 31;
-    const unsigned step = __ldcg(&a.ctl->step);
-    const int ntiles = __ldcg(&a.ctl->ntiles);
+    allow_dependents();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -269,6 +268,9 @@ batch_step_kernel(const BatchArgs a) {
         if (warp < NW) gram_init_full(gram + warp * kGramFullHalves);
     }
     __syncthreads();
+    wait_dependency();
+    const unsigned step = __ldcg(&a.ctl->step);
+    const int ntiles = __ldcg(&a.ctl->ntiles);
 
     const int tbeg = (int)((long long)blockIdx.x * ntiles / gridDim.x);
     const int ntile = (int)((long long)(blockIdx.x + 1) * ntiles / gridDim.x) - tbeg;

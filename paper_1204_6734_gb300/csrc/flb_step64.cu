@@ -22,6 +22,7 @@
 #include <mutex>
 
 #include "flb_step64.cuh"
+#include "flb_tma.cuh"
 
 namespace flb {
 
@@ -90,6 +91,8 @@ __device__ __forceinline__ void add_node(double (&s)[kSums], const double (&g)[9
 // the sums of the nodes that the first one collides.
 template <int BASIS, bool SAMPLE, bool TABLE, bool SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 64 : 32) step64_kernel(const Step64Args a, const CollideConst<double> cc) {
+    allow_dependents();
+    wait_dependency();
     if (SAMPLE && (int)blockIdx.x >= a.blocks) {
         if (a.prev && threadIdx.x < 32) add_partials(a.prev, a.blocks, a.acc, blockIdx.x - a.blocks);
         return;
@@ -145,22 +148,19 @@ std::mutex g_mutex;
 NoiseTables g_tables[kMaxDevices];
 
 template <int BASIS, bool SAMPLE, bool SPLIT>
-void launch(const Step64Args& a, const CollideConst<double>& cc, cudaStream_t s) {
+cudaError_t launch(const Step64Args& a, const CollideConst<double>& cc, cudaStream_t s) {
     const int grid = a.blocks + (SAMPLE ? kSums : 0), threads = SPLIT ? 64 : 32;
-    if (a.noise.radius)
-        step64_kernel<BASIS, SAMPLE, true, SPLIT><<<grid, threads, 0, s>>>(a, cc);
-    else
-        step64_kernel<BASIS, SAMPLE, false, SPLIT><<<grid, threads, 0, s>>>(a, cc);
+    const void* fn = a.noise.radius ? (const void*)step64_kernel<BASIS, SAMPLE, true, SPLIT>
+                                    : (const void*)step64_kernel<BASIS, SAMPLE, false, SPLIT>;
+    void* params[2] = {(void*)&a, (void*)&cc};
+    return launch_dependent(fn, dim3(grid), dim3(threads), params, 0, s);
 }
 
 template <int BASIS>
-void launch(const Step64Args& a, const CollideConst<double>& cc, bool sample, bool split, cudaStream_t s) {
-    if (!sample)
-        launch<BASIS, false, false>(a, cc, s);
-    else if (split)
-        launch<BASIS, true, true>(a, cc, s);
-    else
-        launch<BASIS, true, false>(a, cc, s);
+cudaError_t launch(const Step64Args& a, const CollideConst<double>& cc, bool sample, bool split, cudaStream_t s) {
+    return !sample ? launch<BASIS, false, false>(a, cc, s)
+           : split ? launch<BASIS, true, true>(a, cc, s)
+                   : launch<BASIS, true, false>(a, cc, s);
 }
 
 }  // namespace
@@ -218,13 +218,9 @@ cudaError_t step64(const Step64Args& a, const CollideConst<double>& cc, int basi
     // the launch that added the sums gone as well); with more blocks the FP64
     // pipe is busy either way (400 x 300: 83 %)
     const bool split = a.blocks <= 2 * sms;
-    if (basis == 0)
-        launch<0>(a, cc, sample, split, s);
-    else if (basis == 1)
-        launch<1>(a, cc, sample, split, s);
-    else
-        launch<2>(a, cc, sample, split, s);
-    return cudaGetLastError();
+    return basis == 0   ? launch<0>(a, cc, sample, split, s)
+           : basis == 1 ? launch<1>(a, cc, sample, split, s)
+                        : launch<2>(a, cc, sample, split, s);
 }
 
 cudaError_t step64_flush(const double* partials, int blocks, double* acc, cudaStream_t s) {

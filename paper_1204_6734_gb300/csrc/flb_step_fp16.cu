@@ -76,6 +76,7 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
     __half* gram = reinterpret_cast<__half*>(red + 256);
 
     const int c = threadIdx.x, warp = c >> 5, lane_id = c & 31;
+    allow_dependents();
     if (c == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -88,6 +89,7 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
         gram_init(gram + warp * kGramWarpHalves);
     }
     __syncthreads();
+    wait_dependency();
     const int Lx = a.geo.Lx, Ly = a.geo.Ly;
 
     // thread 0 issues the first tiles; after that the last warp to release a
@@ -262,7 +264,7 @@ cudaError_t fp16_step(const TmaPlan& plan, int src, const HArgs& a, const Collid
     args.tiles_x = plan.tiles_x;
     args.ntiles = plan.ntiles;
     void* params[3] = {(void*)&plan.map[src], (void*)&args, (void*)&cc};
-    return cudaLaunchKernel(fp16_kernel(plan.nw, basis, sample), dim3(plan.grid), dim3(plan.nw * 32), params, plan.smem,
+    return launch_dependent(fp16_kernel(plan.nw, basis, sample), dim3(plan.grid), dim3(plan.nw * 32), params, plan.smem,
                             s);
 }
 

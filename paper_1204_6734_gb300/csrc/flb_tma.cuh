@@ -130,9 +130,36 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// Dependent launches (launch_dependent below): a step kernel lets the next one of
+// the stream start as soon as its own CTAs run -- each CTA of the next takes an
+// SM when this kernel's leaves it, and sets up its barriers there -- and waits,
+// before it touches anything the previous kernel wrote or reads, for that
+// kernel's end. us per step without and with: FP16 store 2000 x 1500 65.6 / 63.1,
+// FP64 400 x 300 131.5 / 128.1 and 32 x 32 16.4 / 15.5, 48 replicas (6.0 M nodes)
+// 152.9 / 151.6. The one-lattice FP32 step does not use it: 4096^2 f-norm 300.1 /
+// 300.0, 2048^2 Hermite norm 61.5 / 62.0.
+__device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_dependency() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Barrier among the first `count` threads of the CTA (named barrier `id`).
 __device__ __forceinline__ void named_sync(int id, int count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// Launch fn so that it may start while the previous kernel of the stream ends
+// (fn calls wait_dependency).
+inline cudaError_t launch_dependent(const void* fn, dim3 grid, dim3 block, void** params, size_t smem, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
 }  // namespace flb
