@@ -136,8 +136,7 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
 // before it touches anything the previous kernel wrote or reads, for that
 // kernel's end. us per step without and with: FP16 store 2000 x 1500 65.6 / 63.1,
 // FP64 400 x 300 131.5 / 128.1 and 32 x 32 16.4 / 15.5, 48 replicas (6.0 M nodes)
-// 152.9 / 151.6. The one-lattice FP32 step does not use it: 4096^2 f-norm 300.1 /
-// 300.0, 2048^2 Hermite norm 61.5 / 62.0.
+// 152.9 / 151.6; the one-lattice FP32 step: flb_step_tma.cu.
 __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_dependency() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
