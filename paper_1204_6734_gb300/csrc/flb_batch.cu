@@ -253,8 +253,9 @@ void plan_resident(flb_batch_s* b, bool sample) {
         return a.nodes != c.nodes ? a.nodes > c.nodes : a.slot < c.slot;
     });
     const int R = (int)v.size();
-    // one launch per step: 8 us, and the padded tiles at the step kernel's rate
-    const double one_step = 8.0 + padded / 44e3;
+    // one launch per step: 5 us (8 sampled), and the padded tiles at the step
+    // kernel's rate
+    const double one_step = (sample ? 8.0 : 5.0) + padded / 44e3;
     const auto smem_of = [&](int64_t cells, int warps) {
         return cells > 1024LL * warps ? kResSmemMax + 1
                                       : kResHotBytes + res_smem_bytes((int)cells, mode, warps);

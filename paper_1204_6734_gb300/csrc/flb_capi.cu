@@ -482,6 +482,13 @@ cudaError_t launch_step_tma(flb_lattice h, bool sample, float* fields) {
     return tma_step(plan, h->cur, a, collide_const<float>(&h->p), h->p.basis, sample, h->stream);
 }
 
+DevCodec dev_codec(flb_lattice h) {
+    DevCodec c;
+    for (int i = 0; i < 9; ++i) c.ref[i] = (float)h->ref[i];
+    c.scale = (float)std::sqrt(h->p.kT);
+    return c;
+}
+
 // How many of the next n steps one resident launch takes (0: none): the kernel
 // is on, the lattice fits, and the stream is not being captured (a mailbox tag
 // may not be replayed). The steps before the first sampled one go by themselves
@@ -494,8 +501,9 @@ int64_t resident_steps(flb_lattice h, int64_t n) {
         const int64_t quiet = h->warmup - h->t;
         if (quiet >= kResMinSteps && n - quiet >= kResMinSteps) n = quiet;
     }
-    if (count_sampled(h->t, h->t + n, h->warmup, h->every) > 0 &&
-        (!h->res.smem[1] || h->tma.sample_mode != kPlanTensorSampling))
+    const bool sample = count_sampled(h->t, h->t + n, h->warmup, h->every) > 0;
+    if (!resident_pays(h->res, (double)h->p.Lx * h->p.Ly, h->p.precision == FLB_FP16_DEV, sample) ||
+        (sample && h->p.precision == FLB_FP32 && h->tma.sample_mode != kPlanTensorSampling))
         return 0;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) {
@@ -509,8 +517,8 @@ cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
     ResidentArgs a;
     std::memset((void*)&a, 0, sizeof(a));
     const int64_t ns = count_sampled(h->t, h->t + n, h->warmup, h->every);
-    a.k.src = (const float*)h->buf[h->cur];
-    a.k.dst = (float*)h->buf[h->cur ^ (n & 1)];
+    a.k.src = h->buf[h->cur];
+    a.k.dst = h->buf[h->cur ^ (n & 1)];
     a.k.geo = h->geo;
     a.k.gx = h->res.gx;
     a.k.gy = h->res.gy;
@@ -536,7 +544,15 @@ cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
         a.ref[i] = (float)h->ref[i];
         a.snref[i] = (float)(-h->ref[i] / a.s);
     }
-    const cudaError_t ce = resident_step(h->res, a, collide_const<float>(&h->p), h->p.basis, ns > 0, h->stream);
+    const bool half = h->p.precision == FLB_FP16_DEV;
+    if (half) {   // the codec of launch_step_fp16
+        const DevCodec c = dev_codec(h);
+        a.scale = c.scale;
+        a.s = c.scale;
+        a.sinv = 1.0f / c.scale;
+        for (int i = 0; i < 9; ++i) a.snref[i] = -c.ref[i] * a.sinv;
+    }
+    const cudaError_t ce = resident_step(h->res, a, collide_const<float>(&h->p), h->p.basis, half, ns > 0, h->stream);
     if (ce == cudaSuccess) {
         h->tag += (uint32_t)n;
         h->nsamp += ns * (int64_t)h->p.Lx * h->p.Ly;
@@ -552,13 +568,6 @@ bool uses_tma(flb_lattice h) {
 
 // Every step but the generic kernel's adds its sums to h->acc itself.
 bool reduces_in_kernel(flb_lattice h) { return uses_tma(h) || h->p.precision != FLB_FP32; }
-
-DevCodec dev_codec(flb_lattice h) {
-    DevCodec c;
-    for (int i = 0; i < 9; ++i) c.ref[i] = (float)h->ref[i];
-    c.scale = (float)std::sqrt(h->p.kT);
-    return c;
-}
 
 // FP16 deviation store: h = (f - ref) / sqrt(kT), collision in FP32.
 cudaError_t launch_step_fp16(flb_lattice h, bool sample) {
@@ -588,6 +597,15 @@ cudaError_t launch_step(flb_lattice h, bool sample, float* fields = nullptr) {
     if (h->p.precision == FLB_FP16_DEV) return launch_step_fp16(h, sample);
     if (uses_tma(h)) return launch_step_tma(h, sample, fields);
     return launch_generic(h, sample);
+}
+
+// The resident launch of a lattice, if it ever pays.
+ResidentPlan plan_resident(const flb_params* p, int sms, bool cut) {
+    if (p->precision == FLB_FP64) return ResidentPlan();
+    const ResidentPlan r = resident_plan(p->Lx, p->Ly, sms, cut);
+    const double nodes = (double)p->Lx * p->Ly;
+    const bool half = p->precision == FLB_FP16_DEV;
+    return resident_pays(r, nodes, half, false) || resident_pays(r, nodes, half, true) ? r : ResidentPlan();
 }
 
 int check_device_error(flb_lattice h) {
@@ -624,18 +642,18 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
         }
         h->ws = (char*)dev_workspace;
         h->own_ws = false;
-        if (p->precision == FLB_FP32) h->res = resident_plan(p->Lx, p->Ly, sms, false);
+        h->res = plan_resident(p, sms, false);
     } else {
         // the mailboxes of a cut lattice are part of the library's own
         // allocation (a caller's workspace keeps its size: the lattice is then
         // not cut)
-        if (p->precision == FLB_FP32) h->res = resident_plan(p->Lx, p->Ly, sms, true);
+        h->res = plan_resident(p, sms, true);
         const size_t mail = 2 * sizeof(uint64_t) * (size_t)h->res.mail_words;
         void* ptr = nullptr;
         if (mail && cudaMalloc(&ptr, L.total + mail) != cudaSuccess) {
             cudaGetLastError();
             ptr = nullptr;
-            h->res = resident_plan(p->Lx, p->Ly, sms, false);
+            h->res = plan_resident(p, sms, false);
         }
         if (!ptr && cudaMalloc(&ptr, L.total) != cudaSuccess) {
             cudaGetLastError();
@@ -712,7 +730,7 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
             h->tma_quiet.ready = false;
         }
     }
-    if (ce == cudaSuccess && h->res.gx && resident_prepare(h->res, p->basis) != cudaSuccess) {
+    if (ce == cudaSuccess && h->res.gx && resident_prepare(h->res, p->basis, p->precision == FLB_FP16_DEV) != cudaSuccess) {
         cudaGetLastError();
         h->res.gx = 0;
     }

@@ -10,37 +10,49 @@ namespace flb {
 
 namespace {
 
+template <class Par>
 const void* kernel_of(int basis, bool sample) {
-    if (basis == 0) return sample ? (const void*)resident_kernel<0, kResStaged> : (const void*)resident_kernel<0, kResQuiet>;
-    if (basis == 1) return sample ? (const void*)resident_kernel<1, kResStaged> : (const void*)resident_kernel<1, kResQuiet>;
-    return sample ? (const void*)resident_kernel<2, kResStaged> : (const void*)resident_kernel<2, kResQuiet>;
+    if (basis == 0)
+        return sample ? (const void*)resident_kernel<0, kResStaged, Par> : (const void*)resident_kernel<0, kResQuiet, Par>;
+    if (basis == 1)
+        return sample ? (const void*)resident_kernel<1, kResStaged, Par> : (const void*)resident_kernel<1, kResQuiet, Par>;
+    return sample ? (const void*)resident_kernel<2, kResStaged, Par> : (const void*)resident_kernel<2, kResQuiet, Par>;
+}
+
+const void* kernel_of(int basis, bool half, bool sample) {
+    return half ? kernel_of<LatticePar16>(basis, sample) : kernel_of<LatticePar>(basis, sample);
 }
 
 // Estimated microseconds of a step (f-norm, no sampling): wp warp passes of 64
 // nodes on the four schedulers of an SM; blocks that exchange add their words'
-// trip through L2 and the passes whose lanes move them (a row on the edge; all
-// rows are edges twice where a block has one; a cut across x puts two edge
-// lanes into every row). Measured: 21 x 21 in one block 1.8, in two 2.1; 64 x 64
-// in 1 / 4 / 16 / 64 blocks 11.1 / 3.4 / 2.0 / 2.7; 300 x 130 in 26 / 44 / 65 /
-// 130 blocks 5.2 / 3.7 / 3.5 / 4.1; 512 x 512 in 128 x 1 7.0, 2 x 74 7.1, 8 x 19
-// 7.9; 4000 x 20 in 1 / 2 / 4 / 7 x 20 20.0 / 10.5 / 5.7 / 4.9; 1000 x 750 in
-// 150 x 1 16.4, 2 x 75 22.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
+// trip through L2 and the passes whose lanes move them (a row on the edge; a
+// block of one row waits at both). A cut across x puts edge lanes into every
+// row, and a warp waits at one edge after the other. Measured: 21 x 21 in one
+// block 1.8, in two 2.1; 64 x 64 in 1 / 4 / 16 / 64 blocks 11.1 / 3.4 / 2.0 / 2.7;
+// 300 x 130 in 26 / 44 / 65 / 130 blocks 5.2 / 3.7 / 3.5 / 4.1, in 2 x 65 4.7, 3 x 43
+// 7.1; 626 x 62 in 1 x 62 4.7, 2 x 62 4.4, 2 x 31 5.5, 7 x 21 7.3; 4000 x 20 in 2 / 4 / 7
+// x 20 10.5 / 5.7 / 5.0; 512 x 512 in 128 blocks 7.0, 2 x 74 7.1; 1000 x 750 in 150
+// 16.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
 }  // namespace
 
 double resident_step_us(int wp, int gx, int gy, int bw, int bh) {
     double t = std::max(1.75, 0.69 * ((wp + 3) / 4) + 0.3);
     if (gy > 1) t += 0.3 + 0.072 * bw / 32.0 + (bh == 1 ? 1.2 : 0.0);   // one row: two waits in a row
-    if (gx > 1) t += 1.0 + 0.08 * std::min(wp, bh);
+    if (gx > 1) t += bh == 1 ? 0.3 : bh == 2 ? 2.3 : 5.0;
     return t;
 }
 
-namespace {
-
-// The same for one launch per step, from the measured 6.2 (up to 300 x 130),
-// 8.2 (400 x 300), 10.3 (512 x 512), 19.8 (1000 x 750), 20.8 (900 x 900);
-// sampled 2 to 4 more.
-double one_step_us(double nodes) { return 6.2 + nodes / 55e3; }
-}  // namespace
+// One launch per step, without / with sampling, measured: FP32 up to 300 x 130
+// 4.0 / 8.0, 400 x 300 6.4 / 10.0, 512 x 512 8.5 / 12.0, 700 x 600 10.3 / 14.2, 1000 x
+// 750 17.8 / 20.5, 900 x 900 19.4 / 22.6; FP16 store 3.4 / 5.9, 5.2 / 7.7, 8.5 / 11.0,
+// 11.0 / 14.2, 15.5 / 20.3, 18.0 / 22.6. Against that this kernel: 300 x 130 3.5 / 4.1,
+// 626 x 62 4.4 / 5.3, 400 x 300 4.2 / 4.9, 512 x 512 7.0 / 8.0, 700 x 600 9.5 / 10.9,
+// 1000 x 750 16.3 / 19.1, 900 x 900 17.6 / 20.7; the FP16 store 3 to 5 % more.
+bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample) {
+    if (!p.gx || !p.smem[sample]) return false;
+    const double us = half ? 1.05 * p.us : p.us, rest = nodes / 54e3;
+    return sample ? 1.12 * us + 0.3 < (half ? 5.9 : 7.9) + rest : us + 0.6 < (half ? 3.4 : 4.0) + rest;
+}
 
 ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
     ResidentPlan best;
@@ -62,6 +74,7 @@ ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
             const double c = resident_step_us(wp, gx, gy, bw, bh);
             if (c >= cost) continue;
             cost = c;
+            best.us = c;
             best.gx = gx;
             best.gy = gy;
             best.threads[0] = warps * 32;
@@ -71,22 +84,21 @@ ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
             best.mail_words = res_mail_words(Lx, Ly, gx, gy);
         }
     }
-    if (cost > one_step_us((double)Lx * Ly)) best = ResidentPlan();
     return best;
 }
 
-cudaError_t resident_prepare(const ResidentPlan& p, int basis) {
+cudaError_t resident_prepare(const ResidentPlan& p, int basis, bool half) {
     cudaError_t ce = cudaSuccess;
     for (int smp = 0; smp < 2 && ce == cudaSuccess; ++smp)
         if (p.smem[smp])
-            ce = cudaFuncSetAttribute(kernel_of(basis, smp), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
+            ce = cudaFuncSetAttribute(kernel_of(basis, half, smp), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
     return ce;
 }
 
 cudaError_t resident_step(const ResidentPlan& p, const ResidentArgs& a, const CollideConst<float>& cc, int basis,
-                          bool sample, cudaStream_t s) {
+                          bool half, bool sample, cudaStream_t s) {
     void* params[2] = {(void*)&a, (void*)&cc};
-    const void* fn = kernel_of(basis, sample);
+    const void* fn = kernel_of(basis, half, sample);
     const dim3 grid(p.gx * p.gy), block(p.threads[sample]);
     // blocks that wait for one another have to be on the GPU together
     if (p.gx * p.gy > 1) return cudaLaunchCooperativeKernel(fn, grid, block, params, p.smem[sample], s);

@@ -72,8 +72,8 @@ __host__ __device__ constexpr size_t res_smem_bytes(int cells, int mode, int war
 
 // One CTA's block of one lattice and what to do with it.
 struct ResBlock {
-    const float* src;       // holds f*(t0 - 1)
-    float* dst;             // receives f*(t0 + n - 1)
+    const void* src;        // holds f*(t0 - 1), in the store's type
+    void* dst;              // receives f*(t0 + n - 1)
     Geometry geo;
     int x0, y0, bw, bh;
     int gx, gy, ix, iy;     // the block's place in the grid of blocks
@@ -134,6 +134,14 @@ __device__ __forceinline__ int res_word(const ResBlock& k, int X, int Y) {
         const int j = In ? wrap(k.ix - cvx(I), k.gx) : k.ix, y0 = k.gy > 1 ? 6 * k.gy * k.geo.Lx : 0;
         return y0 + (((cvx(I) > 0 ? 0 : k.gx) + j) * 3 + res_kx(I)) * k.geo.Ly + (In ? wrap(Y - cvy(I), k.geo.Ly) : Y);
     }
+}
+
+template <class T>
+__device__ __forceinline__ void store_lane(T* p, const Geometry& geo, int x, int y, const f2 f[9], int k) {
+    T v[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = (T)lane(f[i], k);
+    store_node_ghosts(p, geo, x, y, v);
 }
 
 // The nine cells of node A (word offsets, without the population's own offset)
@@ -255,9 +263,11 @@ __device__ __forceinline__ double res_sum(const double* red, int q, double s) {
     return s * s * red[j < 8 ? 8 * i + j : (i < 8 ? 64 + 2 * i : 80)];
 }
 
-// Steps 0..n-1 of one block. Par: the lattice's parameters -- key, cc (the
-// collision constants), s (the Gram scale), scaled(f, i) (the deviation of
-// population i in units of s), ref(i) (f_i^0(rho0, u0)).
+// Steps 0..n-1 of one block. Par: the lattice's parameters -- Store (the type in
+// HBM; the cells hold the stored value as a float), decode(v, i) and encode(f,
+// i) (from and to the stored value; encode rounds to the store), key, cc (the
+// collision constants), s (the Gram scale), scaled(v, i) (the stored value's
+// deviation in units of s), ref(i) (f_i^0(rho0, u0)).
 template <int BASIS, int SAMPLE, class Par>
 __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, unsigned char* smem) {
     float* cell = reinterpret_cast<float*>(smem);
@@ -290,15 +300,17 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
     const int dy = T / bw, dx = T - dy * bw;
     const int ys = c / bw, xs = c - ys * bw;
     const bool cutx = k.gx > 1, cuty = k.gy > 1;
+    using Store = typename Par::Store;
     {
+        const Store* src = static_cast<const Store*>(k.src);
         int x = xs, y = ys;
         for (int m = c; m < pairs; m += T) {
             const int X = k.x0 + x, Y = k.y0 + y, XB = k.x0 + bw - 1 - x, YB = k.y0 + bh - 1 - y;
             float va[9], vb[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                va[i] = k.src[pull_at(k.geo, i, X, Y)];
-                vb[i] = k.src[pull_at(k.geo, i, XB, YB)];
+                va[i] = (float)src[pull_at(k.geo, i, X, Y)];
+                vb[i] = (float)src[pull_at(k.geo, i, XB, YB)];
             }
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
@@ -369,7 +381,9 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
             };
             f2 g[9];
             load(g);
-            if (k.fields && st == 0) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g[i] = par.decode(g[i], i);
+            if (sizeof(Store) == 4 && k.fields && st == 0) {
                 f2 d[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) d[i] = g[i] - f2(par.ref(i));
@@ -408,6 +422,8 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                             gram_stage(gh, h);
                     }
                 }
+#pragma unroll
+                for (int i = 0; i < 9; ++i) gg[i] = par.decode(gg[i], i);
             };
             f2 f[9];
             const uint32_t stt =
@@ -416,9 +432,12 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                 if (inA && (stt & 0xFF)) record_error(k.err, (int)(stt & 0xFF), nodeA, t);
                 if (inB && (stt >> 8)) record_error(k.err, (int)(stt >> 8), nodeB, t);
             }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = par.encode(f[i], i);
             if (last) {
-                if (inA) store_lane_ghosts(k.dst + at(k.geo, 0, X, Y), k.geo, X, Y, f, 0);
-                if (inB) store_lane_ghosts(k.dst + at(k.geo, 0, XB, YB), k.geo, XB, YB, f, 1);
+                Store* dst = static_cast<Store*>(k.dst);
+                if (inA) store_lane(dst + at(k.geo, 0, X, Y), k.geo, X, Y, f, 0);
+                if (inB) store_lane(dst + at(k.geo, 0, XB, YB), k.geo, XB, YB, f, 1);
             } else if (inA) {
 #pragma unroll
                 for (int i = 0; i < 9; ++i) cell[a.a(i)] = f[i].v.x;
@@ -438,6 +457,8 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                 if (smp) {
                     if constexpr (SAMPLE == kResExact)
                         gram_mma_pair(gh, gl, reinterpret_cast<float(&)[8]>(gc));
+                    else if constexpr (sizeof(Store) == 2)
+                        gram_mma_rn(gh, reinterpret_cast<float(&)[8]>(gc));
                     else
                         gram_mma(gh, reinterpret_cast<float(&)[8]>(gc));
                 }
@@ -476,6 +497,7 @@ struct ResidentArgs {
     float ref[9];        // f^0(rho0, u0)
     float sinv;          // 1 / s
     float snref[9];      // -ref / s
+    float scale;         // FP16 store: sqrt(kT)
     double s;            // scale of the staged deviations
 };
 
@@ -490,22 +512,42 @@ __host__ __device__ __forceinline__ void res_place(ResBlock& k, int ix, int iy) 
 }
 
 struct LatticePar {
+    using Store = float;
     const NoiseKey& key;
     const CollideConst<float>& cc;
     const ResidentArgs& a;
     double s;
     __device__ __forceinline__ f2 scaled(f2 f, int i) const { return mad(f, f2(a.sinv), f2(a.snref[i])); }
     __device__ __forceinline__ float ref(int i) const { return a.ref[i]; }
+    __device__ __forceinline__ f2 decode(f2 v, int) const { return v; }
+    __device__ __forceinline__ f2 encode(f2 f, int) const { return f; }
 };
 
-template <int BASIS, int SAMPLE>
+// The FP16 deviation store (flb_step_fp16.cu): stored values h = (f - c) / s, s =
+// sqrt(kT), rounded to FP16 in every step.
+struct LatticePar16 {
+    using Store = __half;
+    const NoiseKey& key;
+    const CollideConst<float>& cc;
+    const ResidentArgs& a;
+    double s;
+    __device__ __forceinline__ f2 scaled(f2 v, int) const { return v; }
+    __device__ __forceinline__ float ref(int i) const { return a.ref[i]; }
+    __device__ __forceinline__ f2 decode(f2 v, int i) const { return mad(v, f2(a.scale), f2(a.ref[i])); }
+    __device__ __forceinline__ f2 encode(f2 f, int i) const {
+        const f2 h = mad(f, f2(a.sinv), f2(a.snref[i]));
+        return f2(__half22float2(__floats2half2_rn(h.v.x, h.v.y)));
+    }
+};
+
+template <int BASIS, int SAMPLE, class Par>
 __global__ void __launch_bounds__(kResMaxWarps * 32, 1)
 resident_kernel(const __grid_constant__ ResidentArgs a, const __grid_constant__ CollideConst<float> cc) {
     extern __shared__ __align__(128) unsigned char res_smem[];
     ResBlock k = a.k;
     const int iy = blockIdx.x / k.gx;
     res_place(k, blockIdx.x - iy * k.gx, iy);
-    resident_run<BASIS, SAMPLE>(k, LatticePar{cc.key, cc, a, a.s}, res_smem);
+    resident_run<BASIS, SAMPLE>(k, Par{cc.key, cc, a, a.s}, res_smem);
 }
 
 // Steps of one launch: at least kResMinSteps (fewer cost less one by one).
@@ -516,6 +558,7 @@ constexpr int kResMaxSteps = 1 << 20;
 struct ResidentPlan {
     int gx = 0, gy = 0;      // 0: no resident launch
     int threads[2] = {0, 0};
+    double us = 0;           // estimated time of a step without sampling
     size_t smem[2] = {0, 0}; // without, with sampling (0: does not fit)
     long long mail_words = 0;
 };
@@ -525,11 +568,13 @@ constexpr size_t kResSmemMax = 227 * 1024;
 // Estimated microseconds of a step of a block of bw x bh nodes, wp warp passes,
 // of a lattice cut into gx x gy blocks.
 double resident_step_us(int wp, int gx, int gy, int bw, int bh);
+// Whether a launch of many steps is faster than one launch per step.
+bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample);
 // Cut a lattice for the given number of SMs; `cut` = false: one block only.
 ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut);
 // Raise the kernels' dynamic shared memory limit (once per plan).
-cudaError_t resident_prepare(const ResidentPlan& p, int basis);
+cudaError_t resident_prepare(const ResidentPlan& p, int basis, bool half);
 cudaError_t resident_step(const ResidentPlan& p, const ResidentArgs& a, const CollideConst<float>& cc, int basis,
-                          bool sample, cudaStream_t s);
+                          bool half, bool sample, cudaStream_t s);
 
 }  // namespace flb

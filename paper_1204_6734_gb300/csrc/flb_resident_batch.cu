@@ -7,6 +7,7 @@ namespace {
 
 template <int SAMPLE>
 struct ReplicaPar {
+    using Store = float;
     const NoiseKey& key;
     const CollidePairs& cc;
     const ReplicaHot& h;
@@ -17,6 +18,8 @@ struct ReplicaPar {
         return SAMPLE == kResExact ? (f - f2(h.ref[i])) * f2(h.sinv) : mad(f, f2(h.sinv), f2(h.snref[i]));
     }
     __device__ __forceinline__ float ref(int i) const { return h.ref[i]; }
+    __device__ __forceinline__ f2 decode(f2 v, int) const { return v; }
+    __device__ __forceinline__ f2 encode(f2 f, int) const { return f; }
 };
 
 template <int BASIS, int SAMPLE>

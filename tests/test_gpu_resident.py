@@ -60,6 +60,20 @@ def test_resident_equals_one_step_per_launch(Lx, Ly, basis):
     close(sums, rsums, 5 * Lx * Ly)
 
 
+@pytest.mark.parametrize("Lx,Ly", [(1, 1), (9, 1), (21, 21), (33, 65), (300, 130), (257, 129), (20, 601)])
+@pytest.mark.parametrize("basis", ["standard", "local", "lut"])
+def test_resident_fp16_store_equals_single_steps(Lx, Ly, basis):
+    """The FP16 store: rounded to FP16 in every step, so bit-identical to calls of
+    one step (which take the one-step kernel)."""
+    p = params(Lx, Ly, basis)
+    p.precision = "fp16dev"
+    f0 = start_state(p)
+    got, sums, _ = run(p, [11], f0=f0)
+    ref, rsums, _ = run(p, [1] * 11, f0=f0)
+    np.testing.assert_array_equal(got, ref)
+    close(sums, rsums, 5 * Lx * Ly)
+
+
 @pytest.mark.parametrize("Lx,Ly", [(21, 21), (64, 64), (300, 130)])
 def test_launch_length_does_not_matter(Lx, Ly):
     p = params(Lx, Ly)
