@@ -207,7 +207,8 @@ int flb_state_difference(flb_lattice a, flb_lattice b, double out[3]);
  * transform them. The first call with every > 0 allocates the library's own
  * device buffers (at most 3 complex and 4 double arrays of Lx*Ly values; FP32
  * power-of-two lattices also 4 float arrays of partial sums and 3 float field
- * arrays), freed by flb_destroy. Errors: FLB_ERR_ARG (negative arguments; a
+ * arrays; where a launch makes many steps, fields and spectra of up to 16
+ * samples, 2^20 nodes in all), freed by flb_destroy. Errors: FLB_ERR_ARG (negative arguments; a
  * side above 20480 in FP32 or 10240 in FP64), FLB_ERR_OOM, a recorded device
  * error (sticky). */
 int flb_set_structure_sampling(flb_lattice h, int64_t warmup, int64_t every);

@@ -513,6 +513,7 @@ int64_t resident_steps(flb_lattice h, int64_t n) {
     return cap == cudaStreamCaptureStatusNone ? n : 0;
 }
 
+// fields: where the structure-factor samples of these steps go, if any.
 cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
     ResidentArgs a;
     std::memset((void*)&a, 0, sizeof(a));
@@ -538,6 +539,12 @@ cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
     a.k.err = h->err;
     a.k.lut = h->lut32;
     a.k.fields = fields;
+    a.k.ffirst = a.k.fevery = n;
+    if (fields) {
+        const int64_t since = h->t - h->sk_warmup;
+        a.k.ffirst = (int)std::min<int64_t>(n, since < 0 ? -since : (h->sk_every - since % h->sk_every) % h->sk_every);
+        a.k.fevery = (int)std::min<int64_t>(h->sk_every, kResMaxSteps);
+    }
     a.s = tensor_sampling_ok(&h->p) ? gram_scale(&h->p) : 1.0;
     a.sinv = (float)(1.0 / a.s);
     for (int i = 0; i < 9; ++i) {
@@ -876,7 +883,8 @@ int flb_set_structure_sampling(flb_lattice h, int64_t warmup, int64_t every) {
     if (h->sticky) return h->sticky;
     if (every > 0 && !h->sk) {
         const int rc = structure_create(&h->sk, h->p.Lx, h->p.Ly,
-                                        h->p.precision == FLB_FP64 ? 8 : 4, h->p.precision == FLB_FP32);
+                                        h->p.precision == FLB_FP64 ? 8 : 4, h->p.precision == FLB_FP32,
+                                        h->res.gx > 0);
         if (rc) return rc;
     }
     h->sk_warmup = warmup;
@@ -912,19 +920,24 @@ int flb_step(flb_lattice h, int64_t n) {
         if (sk_due && !fields)
             ce = structure_sample(h->sk, h->buf[h->cur], h->p.precision, h->geo, dev_codec(h), h->ref,
                                   h->stream);
-        // up to the next structure-factor sample in one launch
+        // in one launch: up to the next structure-factor sample or, where the
+        // launch forms the fields itself, as many samples as their buffer holds
         int64_t run = n - s;
+        float* const many = h->sk_every > 0 && uses_tma(h) ? structure_fields(h->sk) : nullptr;
         if (h->sk_every > 0) {
             const int64_t next = h->t < h->sk_warmup ? h->sk_warmup
                                                      : h->t + h->sk_every - (h->t - h->sk_warmup) % h->sk_every;
-            run = std::min(run, next - h->t);
+            const int64_t more = many ? structure_room(h->sk) - (sk_due ? 1 : 0) : 0;
+            run = next - h->t > run || h->sk_every > run ? std::min(run, next - h->t)
+                                                         : std::min(run, next - h->t + more * h->sk_every);
         }
         run = ce == cudaSuccess ? resident_steps(h, run) : 0;
         if (run > 0) {
-            ce = launch_resident(h, (int)run, fields);
+            const int64_t samples = many ? count_sampled(h->t, h->t + run, h->sk_warmup, h->sk_every) : 0;
+            ce = launch_resident(h, (int)run, samples > 0 ? many : nullptr);
             if (ce == cudaSuccess) {
                 s += run;
-                if (fields) ce = structure_sample_fields(h->sk, h->stream);
+                if (samples > 0) ce = structure_sample_fields(h->sk, (int)samples, h->stream);
                 if (ce != cudaSuccess) return FLB_ERR_CUDA;
                 continue;
             }
@@ -934,7 +947,7 @@ int flb_step(flb_lattice h, int64_t n) {
             ce = cudaSuccess;
         }
         if (ce == cudaSuccess) ce = launch_step(h, sample, fields);
-        if (ce == cudaSuccess && fields) ce = structure_sample_fields(h->sk, h->stream);
+        if (ce == cudaSuccess && fields) ce = structure_sample_fields(h->sk, 1, h->stream);
         if (ce == cudaSuccess && sample && !reduces_in_kernel(h)) {
             accumulate_partials_kernel<<<kSums, 32, 0, h->stream>>>(h->partials, h->nblocks,
                                                                      h->acc);

@@ -86,7 +86,8 @@ struct ResBlock {
     double* acc;
     DevError* err;
     const float* lut;
-    float* fields;          // structure-factor fields of the state at t0 (or null)
+    float* fields;          // structure-factor fields (3 Lx Ly values each) of the states at
+    int ffirst, fevery;     // t0 + ffirst, t0 + ffirst + fevery, ... (or null)
 };
 
 __device__ __forceinline__ uint64_t ld_mail(const uint64_t* p) {
@@ -329,6 +330,7 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
     int sx = 0, sy = 0;              // steps so far modulo bw, bh
     int until = k.first;             // next step to sample
     int nsum = 0;                    // sampled steps so far
+    int funtil = k.fields ? k.ffirst : k.n, nfield = 0;
     bool pending = false;            // the previous step's partials wait in the slots
     for (int st = 0; st < k.n; ++st) {
         const uint32_t t = k.t0 + (uint32_t)st;
@@ -338,6 +340,11 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
         if constexpr (SAMPLE != kResQuiet) {
             if (pending) res_reduce(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
             pending = false;
+        }
+        float* fields = nullptr;
+        if (st == funtil) {
+            fields = k.fields + (size_t)nfield++ * 3 * Lx * k.geo.Ly;
+            funtil = k.fevery > k.n - st ? k.n : st + k.fevery;
         }
         const uint64_t* in = k.mail + (size_t)(st & 1) * k.mail_words;
         uint64_t* out = k.mail + (size_t)((st + 1) & 1) * k.mail_words;
@@ -383,7 +390,7 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
             load(g);
 #pragma unroll
             for (int i = 0; i < 9; ++i) g[i] = par.decode(g[i], i);
-            if (sizeof(Store) == 4 && k.fields && st == 0) {
+            if (sizeof(Store) == 4 && fields) {
                 f2 d[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) d[i] = g[i] - f2(par.ref(i));
@@ -392,13 +399,13 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                 const f2 fy = (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
                 const size_t N = (size_t)Lx * k.geo.Ly;
                 if (inA) {
-                    float* o = k.fields + (size_t)Y * Lx + X;
+                    float* o = fields + (size_t)Y * Lx + X;
                     o[0] = fr.v.x;
                     o[N] = fx.v.x;
                     o[2 * N] = fy.v.x;
                 }
                 if (inB) {
-                    float* o = k.fields + (size_t)YB * Lx + XB;
+                    float* o = fields + (size_t)YB * Lx + XB;
                     o[0] = fr.v.y;
                     o[N] = fx.v.y;
                     o[2 * N] = fy.v.y;

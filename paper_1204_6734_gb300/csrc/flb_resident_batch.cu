@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kResMaxWarps * 32, 1) resident_batch_kernel(co
         k.err = h.err;
         k.lut = a.lut;
         k.fields = nullptr;
+        k.ffirst = k.fevery = n;
         resident_run<BASIS, SAMPLE>(k, ReplicaPar<SAMPLE>{h.cc.key, h.pc, h, (double)h.gram_s}, res_smem + kResHotBytes);
     }
     // the last CTA to finish advances the batch step (every CTA read it at its start)

@@ -108,16 +108,24 @@ def test_invalid_node_is_reported(Lx, Ly):
     assert where[0] == where[1] == 0
 
 
-def test_structure_samples_between_launches():
-    p = params(64, 32)
+@pytest.mark.parametrize("Lx,Ly,warmup,every,cuts", [
+    (64, 32, 1, 4, [18]),               # several samples left by one launch
+    (64, 32, 0, 3, [7, 50, 1, 42]),     # more than the buffers and the partial sums hold
+    (256, 128, 2, 1, [40]),
+    (32, 512, 5, 7, [3, 3, 30]),
+    (21, 30, 1, 4, [18]),               # a side that is no power of two: one sample at a time
+])
+def test_structure_samples_of_long_launches(Lx, Ly, warmup, every, cuts):
+    p = params(Lx, Ly)
     out = []
     for kernel in (None, "pipelined"):
         with flb.Lattice(p, kernel=kernel) as lat:
-            lat.set_structure_sampling(1, 4)
-            lat.step(18)
-            out.append(lat.structure_factors())
-    assert out[0][3] == out[1][3] == 5
-    for a, b in zip(out[0][:3], out[1][:3]):
+            lat.set_structure_sampling(warmup, every)
+            for n in cuts:
+                lat.step(n)
+            out.append(lat.structure_factors() + (lat.populations(),))
+    assert out[0][3] == out[1][3] == len(range(warmup, sum(cuts), every))
+    for a, b in zip(out[0][:3] + out[0][4:], out[1][:3] + out[1][4:]):
         np.testing.assert_array_equal(a, b)
 
 
