@@ -18,6 +18,14 @@
 // threads in a step, one barrier per step orders the steps, and the wrap of
 // the offsets is the periodic boundary where the lattice is not cut.
 //
+// Cells are addressed in bytes of shared memory: a pair's three column and three
+// row offsets (each the smaller of two unsigned sums) give its 18 addresses by
+// one addition or subtraction each, and what rarely is asked for (a node's place
+// in the lattice) is divided out where it is. As word indices into an array
+// the same took 16.1 instructions per node against 12.4 in the one-step kernel;
+// us per step before and after: 21 x 21 2.18 / 2.08, 300 x 130 4.27 / 4.13, 1000 x 750
+// 16.4 / 15.7, 384 x 21^2 6.25 / 5.90.
+//
 // Node pairs (packed FP32x2): node A is the m-th of the block, node B the m-th
 // from its end, i.e. (bw - 1 - x, bh - 1 - y), so B's cells follow from A's
 // by one subtraction each (cell_i(B) = nn - 1 - cell_opposite(i)(A)), and the
@@ -145,23 +153,66 @@ __device__ __forceinline__ void store_lane(T* p, const Geometry& geo, int x, int
     store_node_ghosts(p, geo, x, y, v);
 }
 
-// The nine cells of node A (word offsets, without the population's own offset)
-// from its row and column offsets, and node B's from them.
+// Shared-memory cells by 32-bit address; population I of a cell is 4 I bytes in.
+template <int I>
+__device__ __forceinline__ float cell_load(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(4 * I) : "memory");
+    return v;
+}
+template <int I>
+__device__ __forceinline__ void cell_store(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0+%1], %2;" ::"r"(a), "n"(4 * I), "f"(v) : "memory");
+}
+
+// The nine cells of node A from its column and row offsets (bytes; the columns
+// hold the address of cell 0), and node B's from them.
 struct ResCells {
-    int r[3], c[3];   // index v + 1
-    int kb;           // 9 (nn - 1)
-    __device__ __forceinline__ int a(int i) const { return r[cvy(i) + 1] + c[cvx(i) + 1] + i; }
-    __device__ __forceinline__ int b(int i) const {
-        return kb - (r[1 - cvy(i)] + c[1 - cvx(i)]) + i;
-    }
+    uint32_t r[3], c[3];   // index v + 1
+    uint32_t kb;           // twice the address of cell 0, plus 36 (nn - 1)
+    template <int I>
+    __device__ __forceinline__ uint32_t a() const { return r[cvy(I) + 1] + c[cvx(I) + 1]; }
+    template <int I>
+    __device__ __forceinline__ uint32_t b() const { return kb - (r[1 - cvy(I)] + c[1 - cvx(I)]); }
+    template <int I>
+    __device__ __forceinline__ f2 load() const { return f2(cell_load<I>(a<I>()), cell_load<I>(b<I>())); }
 };
+
+__device__ __forceinline__ void load_cells(const ResCells& a, f2 (&g)[9]) {
+    g[0] = a.load<0>();
+    g[1] = a.load<1>();
+    g[2] = a.load<2>();
+    g[3] = a.load<3>();
+    g[4] = a.load<4>();
+    g[5] = a.load<5>();
+    g[6] = a.load<6>();
+    g[7] = a.load<7>();
+    g[8] = a.load<8>();
+}
+
+template <int I>
+__device__ __forceinline__ void store_cell(const ResCells& a, const f2 (&f)[9], bool both) {
+    cell_store<I>(a.a<I>(), f[I].v.x);
+    if (both) cell_store<I>(a.b<I>(), f[I].v.y);
+}
+__device__ __forceinline__ void store_cells(const ResCells& a, const f2 (&f)[9], bool both) {
+    store_cell<0>(a, f, both);
+    store_cell<1>(a, f, both);
+    store_cell<2>(a, f, both);
+    store_cell<3>(a, f, both);
+    store_cell<4>(a, f, both);
+    store_cell<5>(a, f, both);
+    store_cell<6>(a, f, both);
+    store_cell<7>(a, f, both);
+    store_cell<8>(a, f, both);
+}
 
 // Receive across one edge: A's populations I0, I1, I2 and B's opposite ones,
 // into the pair's own cells, once all carry the step's tag. skip1, skip2: I1,
 // I2 cross the other axis' boundary, too, and came from there.
 template <int AXIS, int I0, int I1, int I2>
 __device__ __noinline__ void res_receive(const ResBlock& k, const uint64_t* in, uint32_t tag, uint32_t t, int X, int Y,
-                                         int XB, int YB, float* cell, const ResCells& a, bool skip1, bool skip2,
+                                         int XB, int YB, const ResCells& a, bool skip1, bool skip2,
                                          volatile int* gave_up) {
     const uint64_t* pa0 = in + res_word<AXIS, I0, true>(k, X, Y);
     const uint64_t* pa1 = in + res_word<AXIS, I1, true>(k, X, Y);
@@ -194,15 +245,15 @@ __device__ __noinline__ void res_receive(const ResBlock& k, const uint64_t* in, 
             break;
         }
     }
-    cell[a.a(I0)] = __uint_as_float((uint32_t)a0);
-    cell[a.b(opposite(I0))] = __uint_as_float((uint32_t)b0);
+    cell_store<I0>(a.a<I0>(), __uint_as_float((uint32_t)a0));
+    cell_store<opposite(I0)>(a.b<opposite(I0)>(), __uint_as_float((uint32_t)b0));
     if (!skip1) {
-        cell[a.a(I1)] = __uint_as_float((uint32_t)a1);
-        cell[a.b(opposite(I1))] = __uint_as_float((uint32_t)b1);
+        cell_store<I1>(a.a<I1>(), __uint_as_float((uint32_t)a1));
+        cell_store<opposite(I1)>(a.b<opposite(I1)>(), __uint_as_float((uint32_t)b1));
     }
     if (!skip2) {
-        cell[a.a(I2)] = __uint_as_float((uint32_t)a2);
-        cell[a.b(opposite(I2))] = __uint_as_float((uint32_t)b2);
+        cell_store<I2>(a.a<I2>(), __uint_as_float((uint32_t)a2));
+        cell_store<opposite(I2)>(a.b<opposite(I2)>(), __uint_as_float((uint32_t)b2));
     }
 }
 
@@ -210,14 +261,14 @@ __device__ __noinline__ void res_receive(const ResBlock& k, const uint64_t* in, 
 // opposite ones, read back from the pair's cells.
 template <int AXIS, int I0, int I1, int I2>
 __device__ __noinline__ void res_send(const ResBlock& k, uint64_t* out, uint32_t tag, int X, int Y, int XB, int YB,
-                                      const float* cell, const ResCells& a, bool skip1, bool skip2, bool both) {
-    st_mail(out + res_word<AXIS, I0, false>(k, X, Y), cell[a.a(I0)], tag);
-    if (!skip1) st_mail(out + res_word<AXIS, I1, false>(k, X, Y), cell[a.a(I1)], tag);
-    if (!skip2) st_mail(out + res_word<AXIS, I2, false>(k, X, Y), cell[a.a(I2)], tag);
+                                      const ResCells& a, bool skip1, bool skip2, bool both) {
+    st_mail(out + res_word<AXIS, I0, false>(k, X, Y), cell_load<I0>(a.a<I0>()), tag);
+    if (!skip1) st_mail(out + res_word<AXIS, I1, false>(k, X, Y), cell_load<I1>(a.a<I1>()), tag);
+    if (!skip2) st_mail(out + res_word<AXIS, I2, false>(k, X, Y), cell_load<I2>(a.a<I2>()), tag);
     if (!both) return;
-    st_mail(out + res_word<AXIS, opposite(I0), false>(k, XB, YB), cell[a.b(opposite(I0))], tag);
-    if (!skip1) st_mail(out + res_word<AXIS, opposite(I1), false>(k, XB, YB), cell[a.b(opposite(I1))], tag);
-    if (!skip2) st_mail(out + res_word<AXIS, opposite(I2), false>(k, XB, YB), cell[a.b(opposite(I2))], tag);
+    st_mail(out + res_word<AXIS, opposite(I0), false>(k, XB, YB), cell_load<opposite(I0)>(a.b<opposite(I0)>()), tag);
+    if (!skip1) st_mail(out + res_word<AXIS, opposite(I1), false>(k, XB, YB), cell_load<opposite(I1)>(a.b<opposite(I1)>()), tag);
+    if (!skip2) st_mail(out + res_word<AXIS, opposite(I2), false>(k, XB, YB), cell_load<opposite(I2)>(a.b<opposite(I2)>()), tag);
 }
 
 // A warp's FP32 partials of one step, in the order of the kept entries (C is
@@ -327,7 +378,13 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
         }
     }
 
-    int sx = 0, sy = 0;              // steps so far modulo bw, bh
+    // in bytes: a row of cells, all cells; the steps between a thread's pairs; the
+    // steps so far modulo the block
+    const uint32_t row = 36u * bw, all = row * bh, cell0 = smem_u32(cell);
+    const uint32_t dxo = 36u * dx, dyo = row * dy, dnode = (uint32_t)dx + (uint32_t)Lx * (uint32_t)dy;
+    const uint32_t node0 = (uint32_t)k.x0 + (uint32_t)Lx * (uint32_t)k.y0;
+    const uint32_t nodes = 2u * node0 + (uint32_t)(bw - 1) + (uint32_t)Lx * (uint32_t)(bh - 1);   // A's plus B's
+    uint32_t sx = 0, sy = 0;
     int until = k.first;             // next step to sample
     int nsum = 0;                    // sampled steps so far
     int funtil = k.fields ? k.ffirst : k.n, nfield = 0;
@@ -348,39 +405,44 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
         }
         const uint64_t* in = k.mail + (size_t)(st & 1) * k.mail_words;
         uint64_t* out = k.mail + (size_t)((st + 1) & 1) * k.mail_words;
-        int x = xs, y = ys;
+        // node A's column and row as byte offsets, and its number in the lattice
+        uint32_t xo = 36u * xs, yo = row * ys, node = node0 + (uint32_t)xs + (uint32_t)Lx * (uint32_t)ys;
         for (int m0 = warp * 32; m0 < pairs; m0 += T) {
             const int m = m0 + lane_id;
             const bool inA = m < pairs, inB = inA && 2 * m != nn - 1;
+            // the offsets less the steps so far, modulo the block (unsigned: the
+            // one that has not wrapped is the smaller one)
             ResCells a;
-            {
-                int cp = x - sx, cm = x + sx, rp = y - sy, rm = y + sy;
-                cp += cp < 0 ? bw : 0;
-                cm -= cm >= bw ? bw : 0;
-                rp += rp < 0 ? bh : 0;
-                rm -= rm >= bh ? bh : 0;
-                a.c[0] = 9 * cm;
-                a.c[1] = 9 * x;
-                a.c[2] = 9 * cp;
-                a.r[0] = 9 * bw * rm;
-                a.r[1] = 9 * bw * y;
-                a.r[2] = 9 * bw * rp;
-                a.kb = 9 * (nn - 1);
-            }
-            const int X = k.x0 + x, Y = k.y0 + y, XB = k.x0 + bw - 1 - x, YB = k.y0 + bh - 1 - y;
-            const ResEdge e{cutx && x == 0, cutx && x == bw - 1, cuty && y == 0, cuty && y == bh - 1};
+            a.c[0] = cell0 + min(xo + sx, xo + sx - row);
+            a.c[1] = cell0 + xo;
+            a.c[2] = cell0 + min(xo - sx, xo - sx + row);
+            a.r[0] = min(yo + sy, yo + sy - all);
+            a.r[1] = yo;
+            a.r[2] = min(yo - sy, yo - sy + all);
+            a.kb = 2u * cell0 + all - 36u;
+            const uint32_t nodeA = node, nodeB = nodes - node;
+            // places in the lattice, where they are needed
+            const auto place = [&](int& X, int& Y, int& XB, int& YB) {
+                const int x = (int)(xo / 36u), y = (int)(yo / row);
+                X = k.x0 + x;
+                Y = k.y0 + y;
+                XB = k.x0 + bw - 1 - x;
+                YB = k.y0 + bh - 1 - y;
+            };
+            const ResEdge e{cutx && xo == 0, cutx && xo == row - 36u, cuty && yo == 0, cuty && yo == all - row};
             const bool edge = inA && e.any();
             if (edge && st > 0) {   // what comes across the cut: into this thread's own cells
                 const uint32_t tag = k.tag0 + (uint32_t)st;
-                if (e.b) res_receive<1, 2, 5, 6>(k, in, tag, t, X, Y, XB, YB, cell, a, false, false, gave_up);
-                if (e.t) res_receive<1, 4, 7, 8>(k, in, tag, t, X, Y, XB, YB, cell, a, false, false, gave_up);
-                if (e.l) res_receive<0, 1, 5, 8>(k, in, tag, t, X, Y, XB, YB, cell, a, e.b, e.t, gave_up);
-                if (e.r) res_receive<0, 3, 7, 6>(k, in, tag, t, X, Y, XB, YB, cell, a, e.t, e.b, gave_up);
+                int X, Y, XB, YB;
+                place(X, Y, XB, YB);
+                if (e.b) res_receive<1, 2, 5, 6>(k, in, tag, t, X, Y, XB, YB, a, false, false, gave_up);
+                if (e.t) res_receive<1, 4, 7, 8>(k, in, tag, t, X, Y, XB, YB, a, false, false, gave_up);
+                if (e.l) res_receive<0, 1, 5, 8>(k, in, tag, t, X, Y, XB, YB, a, e.b, e.t, gave_up);
+                if (e.r) res_receive<0, 3, 7, 6>(k, in, tag, t, X, Y, XB, YB, a, e.t, e.b, gave_up);
             }
-            auto load = [&](f2* g) {
+            auto load = [&](f2(&g)[9]) {
                 if (inA) {
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) g[i] = f2(cell[a.a(i)], cell[a.b(i)]);
+                    load_cells(a, g);
                 } else {   // a lane past the end: any valid state
 #pragma unroll
                     for (int i = 0; i < 9; ++i) g[i] = f2(1.f);
@@ -398,6 +460,8 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                 const f2 fx = (d[1] - d[3]) + ((d[5] - d[6]) + (d[8] - d[7]));
                 const f2 fy = (d[2] - d[4]) + ((d[5] + d[6]) - (d[7] + d[8]));
                 const size_t N = (size_t)Lx * k.geo.Ly;
+                int X, Y, XB, YB;
+                place(X, Y, XB, YB);
                 if (inA) {
                     float* o = fields + (size_t)Y * Lx + X;
                     o[0] = fr.v.x;
@@ -411,9 +475,8 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                     o[2 * N] = fy.v.y;
                 }
             }
-            const uint32_t nodeA = (uint32_t)X + (uint32_t)Lx * (uint32_t)Y;
-            const uint32_t nodeB = (uint32_t)XB + (uint32_t)Lx * (uint32_t)YB;
-            auto refetch = [&](f2* gg) {
+            auto refetch = [&](f2* out9) {
+                f2(&gg)[9] = *reinterpret_cast<f2(*)[9]>(out9);
                 load(gg);
                 if constexpr (SAMPLE != kResQuiet) {
                     if (smp) {
@@ -443,20 +506,20 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
             for (int i = 0; i < 9; ++i) f[i] = par.encode(f[i], i);
             if (last) {
                 Store* dst = static_cast<Store*>(k.dst);
+                int X, Y, XB, YB;
+                place(X, Y, XB, YB);
                 if (inA) store_lane(dst + at(k.geo, 0, X, Y), k.geo, X, Y, f, 0);
                 if (inB) store_lane(dst + at(k.geo, 0, XB, YB), k.geo, XB, YB, f, 1);
             } else if (inA) {
-#pragma unroll
-                for (int i = 0; i < 9; ++i) cell[a.a(i)] = f[i].v.x;
-                if (inB)
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) cell[a.b(i)] = f[i].v.y;
+                store_cells(a, f, inB);
                 if (edge) {
                     const uint32_t tag = k.tag0 + (uint32_t)st + 1u;
-                    if (e.t) res_send<1, 2, 5, 6>(k, out, tag, X, Y, XB, YB, cell, a, false, false, inB);
-                    if (e.b) res_send<1, 4, 7, 8>(k, out, tag, X, Y, XB, YB, cell, a, false, false, inB);
-                    if (e.r) res_send<0, 1, 5, 8>(k, out, tag, X, Y, XB, YB, cell, a, e.t, e.b, inB);
-                    if (e.l) res_send<0, 3, 7, 6>(k, out, tag, X, Y, XB, YB, cell, a, e.b, e.t, inB);
+                    int X, Y, XB, YB;
+                    place(X, Y, XB, YB);
+                    if (e.t) res_send<1, 2, 5, 6>(k, out, tag, X, Y, XB, YB, a, false, false, inB);
+                    if (e.b) res_send<1, 4, 7, 8>(k, out, tag, X, Y, XB, YB, a, false, false, inB);
+                    if (e.r) res_send<0, 1, 5, 8>(k, out, tag, X, Y, XB, YB, a, e.t, e.b, inB);
+                    if (e.l) res_send<0, 3, 7, 6>(k, out, tag, X, Y, XB, YB, a, e.b, e.t, inB);
                 }
             }
             // after the stores: what the neighbours wait for leaves first
@@ -470,11 +533,13 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                         gram_mma(gh, reinterpret_cast<float(&)[8]>(gc));
                 }
             }
-            x += dx;
-            y += dy;
-            if (x >= bw) {
-                x -= bw;
-                ++y;
+            xo += dxo;
+            yo += dyo;
+            node += dnode;
+            if (xo >= row) {
+                xo -= row;
+                yo += row;
+                node += (uint32_t)(Lx - bw);
             }
         }
         if constexpr (SAMPLE != kResQuiet) {
@@ -485,8 +550,8 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
                 pending = true;
             }
         }
-        sx = sx + 1 == bw ? 0 : sx + 1;
-        sy = sy + 1 == bh ? 0 : sy + 1;
+        sx = sx + 36u == row ? 0u : sx + 36u;
+        sy = sy + row == all ? 0u : sy + row;
         if (!last) __syncthreads();
     }
     if constexpr (SAMPLE != kResQuiet) {
