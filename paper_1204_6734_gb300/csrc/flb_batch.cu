@@ -512,12 +512,10 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     for (int v = 0; v < kNumBatchVariants && ce == cudaSuccess; ++v)
         for (int smp = 0; smp < 2 && ce == cudaSuccess; ++smp) {
             const void* fn = kernel_of(b->basis, v, smp);
-            ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)batch_smem_bytes(v));
+            ce = allow_smem(fn, batch_smem_bytes(v));
         }
     for (int m2 = 0; m2 < 3 && ce == cudaSuccess; ++m2)
-        ce = cudaFuncSetAttribute(resident_batch_kernel_for(b->basis, m2), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kResSmemMax);
+        ce = allow_smem(resident_batch_kernel_for(b->basis, m2), kResSmemMax);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(b->stream);
     if (ce != cudaSuccess) {
         cudaGetLastError();

@@ -6,12 +6,45 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <mutex>
+#include <vector>
 
 #include "../../include/flb.h"
 #include "flb_device.cuh"
 #include "flb_kernels.cuh"
 
 namespace flb {
+
+// Raise a kernel's dynamic shared memory limit on the current device to `bytes`,
+// unless an earlier call has: creating a lattice asked the runtime two dozen
+// times, about a third of the 230 us it took.
+inline cudaError_t allow_smem(const void* fn, size_t bytes) {
+    struct Done {
+        int dev;
+        const void* fn;
+        size_t bytes;
+    };
+    static std::mutex mutex;
+    static std::vector<Done> done;
+    int dev = 0;
+    cudaError_t ce = cudaGetDevice(&dev);
+    if (ce != cudaSuccess) return ce;
+    std::lock_guard<std::mutex> lock(mutex);
+    Done* mine = nullptr;
+    for (Done& d : done)
+        if (d.dev == dev && d.fn == fn) mine = &d;
+    if (mine && mine->bytes >= bytes) return cudaSuccess;
+    ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (ce != cudaSuccess) return ce;
+    try {
+        if (mine)
+            mine->bytes = bytes;
+        else
+            done.push_back({dev, fn, bytes});
+    } catch (const std::bad_alloc&) {   // asked again next time
+    }
+    return cudaSuccess;
+}
 
 // f_i^0(rho, u) of Eq. d2q9f0.
 inline void feq_host(double rho, double ux, double uy, double f[9]) {

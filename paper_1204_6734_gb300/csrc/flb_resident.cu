@@ -4,6 +4,7 @@
 
 #include <algorithm>
 
+#include "flb_host.h"
 #include "flb_resident.cuh"
 
 namespace flb {
@@ -91,7 +92,7 @@ cudaError_t resident_prepare(const ResidentPlan& p, int basis, bool half) {
     cudaError_t ce = cudaSuccess;
     for (int smp = 0; smp < 2 && ce == cudaSuccess; ++smp)
         if (p.smem[smp])
-            ce = cudaFuncSetAttribute(kernel_of(basis, half, smp), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax);
+            ce = allow_smem(kernel_of(basis, half, smp), kResSmemMax);
     return ce;
 }
 

@@ -24,6 +24,7 @@
 
 #include "flb_collide.cuh"
 #include "flb_gram.cuh"
+#include "flb_host.h"
 #include "flb_internal.h"
 #include "flb_pipeline.cuh"
 #include "flb_tma.cuh"
@@ -244,8 +245,7 @@ cudaError_t fp16_plan(TmaPlan* plan, void* buf0, void* buf1, const Geometry& g) 
     const size_t smem = nw == 8 ? HShape<8>::smem_bytes() : HShape<16>::smem_bytes();
     for (int basis = 0; basis < 3 && ce == cudaSuccess; ++basis)
         for (int smp = 0; smp < 2 && ce == cudaSuccess; ++smp)
-            ce = cudaFuncSetAttribute(fp16_kernel(nw, basis, smp), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem);
+            ce = allow_smem(fp16_kernel(nw, basis, smp), smem);
     if (ce != cudaSuccess) return ce;
     plan->nw = nw;
     plan->smem = smem;

@@ -28,6 +28,7 @@
 
 #include "flb_collide.cuh"
 #include "flb_gram.cuh"
+#include "flb_host.h"
 #include "flb_internal.h"
 #include "flb_pipeline.cuh"
 #include "flb_tma.cuh"
@@ -178,6 +179,7 @@ static_assert(TileShape<8>::smem_bytes() + gram_smem_bytes<8>() <= kMaxSmem, "8 
 static_assert(TileShape<12>::smem_bytes() + gram_smem_bytes<12>() <= kMaxSmem, "12 warps");
 static_assert(TileShape<14>::smem_bytes() + gram_smem_bytes<14>() <= kMaxSmem, "14 warps");
 static_assert(TileShape<16>::smem_bytes() + gram_smem_bytes<16>() <= kMaxSmem, "16 warps");
+static_assert(2 * TileShape<8>::smem_bytes() > kMaxSmem, "one CTA per SM");
 
 // Warp roles. kNoSampling: NW consumer warps + one producer warp.
 // kSamplerWarps: NW consumers + kSamplers sampler warps (sampler w reads rows
@@ -617,25 +619,15 @@ cudaError_t tma_plan(TmaPlan* plan, void* buf0, void* buf1, const Geometry& g, i
     int dev = 0, sms = 0;
     cudaError_t ce = cudaGetDevice(&dev);
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int per_sm = 2;
     for (int basis = 0; basis < 3 && ce == cudaSuccess; ++basis)
-        for (int mode = 0; mode < 4 && ce == cudaSuccess; ++mode) {
-            const void* fn = kernel_for(nw, basis, mode);
-            if (!fn) continue;
-            ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            int n = 0;
-            if (ce == cudaSuccess)
-                ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, warps_for(nw, mode) * 32,
-                                                                   smem);
-            if (n < per_sm) per_sm = n;
-        }
+        for (int mode = 0; mode < 4 && ce == cudaSuccess; ++mode)
+            if (const void* fn = kernel_for(nw, basis, mode)) ce = allow_smem(fn, smem);
     if (ce != cudaSuccess) return ce;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
     plan->nw = nw;
     plan->smem = smem;
     plan->tiles_x = (g.Lx + kTW - 1) / kTW;
     plan->ntiles = plan->tiles_x * ((g.Ly + th - 1) / th);
-    int grid = sms * per_sm;
+    int grid = sms;   // one CTA per SM: no two fit its shared memory
     if (grid > plan->ntiles) grid = plan->ntiles;
     plan->grid = grid < 1 ? 1 : grid;
     if (plan->sample_mode != kSamplerWarps && plan->sample_mode != kFusedSampling &&
