@@ -37,6 +37,35 @@ __device__ __forceinline__ Draw philox_rk(uint32_t c0, uint32_t c1, uint32_t c2,
     return Draw{c0, c1, c2, c3};
 }
 
+// Round keys in shared memory, two to a load: the resident batch kernel (384
+// copies of 21 x 21 5.89 -> 5.80 us per step; the one-step batch kernel, short of
+// registers, spills with them, 151.3 -> 162.6, and loads them one by one).
+struct KeyPairs {
+    const uint2* rk;
+    uint32_t replica;
+    __device__ __forceinline__ explicit KeyPairs(const NoiseKey& k)
+        : rk(reinterpret_cast<const uint2*>(k.rk)), replica(k.replica) {}
+};
+__device__ __forceinline__ Draw philox_rk(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, const KeyPairs& key) {
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const uint2 k = key.rk[r];
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
+        const uint32_t y0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.x;
+        const uint32_t y2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.y;
+        c0 = y0;
+        c1 = (uint32_t)p1;
+        c2 = y2;
+        c3 = (uint32_t)p0;
+    }
+    return Draw{c0, c1, c2, c3};
+}
+template <class K>
+__device__ __forceinline__ void node_fields_of(const K& key, uint32_t node, uint32_t step, uint32_t k[6]) {
+    draw_fields(philox_rk(node, step, key.replica, 0u, key), k);
+}
+
 // Counter (node, step, replica, 0), key = seed.
 __device__ __forceinline__ void node_fields(const NoiseKey& key, uint32_t node, uint32_t step,
                                             uint32_t k[6]) {
@@ -109,14 +138,15 @@ struct NodeNoise {
     }
 };
 
-struct PairNoise {
-    const NoiseKey& key;
+template <class Key>
+struct PairNoiseT {
+    Key key;
     uint32_t nodeA, nodeB, step;
     template <class CC>
     __device__ __forceinline__ void scaled(f2 rho, const CC& cc, f2 n[6]) const {
         uint32_t ka[6], kb[6];
-        node_fields(key, nodeA, step, ka);
-        node_fields(key, nodeB, step, kb);
+        node_fields_of(key, nodeA, step, ka);
+        node_fields_of(key, nodeB, step, kb);
         const f2 nr = rho * f2(-kLn2x2);
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
@@ -132,6 +162,8 @@ struct PairNoise {
         }
     }
 };
+
+using PairNoise = PairNoiseT<const NoiseKey&>;
 
 // xi^a N^a, a = 3..8: FP32 folds the amplitudes into the draw (NodeNoise,
 // PairNoise); FP64 scales unit normals (the arithmetic of the oracle's order).

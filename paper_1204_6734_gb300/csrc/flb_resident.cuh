@@ -497,7 +497,7 @@ __device__ __forceinline__ void resident_run(const ResBlock& k, const Par& par, 
             };
             f2 f[9];
             const uint32_t stt =
-                collide_basis<f2, BASIS>(g, PairNoise{par.key, nodeA, nodeB, t}, refetch, k.lut, par.cc, f);
+                collide_basis<f2, BASIS>(g, PairNoiseT<typename Par::Key>{par.key, nodeA, nodeB, t}, refetch, k.lut, par.cc, f);
             if (stt) {
                 if (inA && (stt & 0xFF)) record_error(k.err, (int)(stt & 0xFF), nodeA, t);
                 if (inB && (stt >> 8)) record_error(k.err, (int)(stt >> 8), nodeB, t);
@@ -585,6 +585,7 @@ __host__ __device__ __forceinline__ void res_place(ResBlock& k, int ix, int iy) 
 
 struct LatticePar {
     using Store = float;
+    using Key = const NoiseKey&;
     const NoiseKey& key;
     const CollideConst<float>& cc;
     const ResidentArgs& a;
@@ -599,6 +600,7 @@ struct LatticePar {
 // sqrt(kT), rounded to FP16 in every step.
 struct LatticePar16 {
     using Store = __half;
+    using Key = const NoiseKey&;
     const NoiseKey& key;
     const CollideConst<float>& cc;
     const ResidentArgs& a;

@@ -8,7 +8,8 @@ namespace {
 template <int SAMPLE>
 struct ReplicaPar {
     using Store = float;
-    const NoiseKey& key;
+    using Key = KeyPairs;
+    KeyPairs key;
     const CollidePairs& cc;
     const ReplicaHot& h;
     double s;
@@ -64,7 +65,7 @@ __global__ void __launch_bounds__(kResMaxWarps * 32, 1) resident_batch_kernel(co
         k.lut = a.lut;
         k.fields = nullptr;
         k.ffirst = k.fevery = n;
-        resident_run<BASIS, SAMPLE>(k, ReplicaPar<SAMPLE>{h.cc.key, h.pc, h, (double)h.gram_s}, res_smem + kResHotBytes);
+        resident_run<BASIS, SAMPLE>(k, ReplicaPar<SAMPLE>{KeyPairs(h.cc.key), h.pc, h, (double)h.gram_s}, res_smem + kResHotBytes);
     }
     // the last CTA to finish advances the batch step (every CTA read it at its start)
     if (threadIdx.x == 0) {
