@@ -57,6 +57,7 @@ bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample) 
 
 ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
     ResidentPlan best;
+    if (36LL * Lx * Ly > (long long)(cut ? sms : 1) * (long long)kResSmemMax) return best;
     double cost = 1e30;
     const int gxmax = cut ? std::min(Lx, sms) : 1;
     for (int gx = 1; gx <= gxmax; ++gx) {
