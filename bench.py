@@ -31,25 +31,25 @@ BYTES_PER_NODE = {"fp32": 72, "fp64": 144}
 # DRAM bytes (read + write) per launch of the FP32 step kernel at 4096^2,
 # f-norm basis, sampling every step (tensor-core sums, 12 colliding warps):
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one 2048^2 launch of
-# the same kernel (156.3 + 101.4 MB) times the 4x nodes; a full-size capture
+# the same kernel (156.0 + 99.7 MB) times the 4x nodes; a full-size capture
 # may take only the launch list. Valid only for the kernel version it was
 # taken on.
-DRAM_TRAFFIC = {("fp32", "local", 4096): 4 * (156.00e6 + 101.18e6),
-                ("fp32", "lut", 4096): 4 * (156.00e6 + 102.08e6)}
+DRAM_TRAFFIC = {("fp32", "local", 4096): 4 * (156.00e6 + 99.70e6),
+                ("fp32", "lut", 4096): 4 * (156.00e6 + 98.73e6)}
 TRAFFIC_SOURCE = "ncu dram bytes of a 2048^2 launch of the same kernel, x 4 (the nodes)"
 # FP64 operations per node-step of the FP64 step kernel (f-norm, sampling
 # every step): 2 DFMA + DADD + DMUL thread instructions counted by ncu on a
-# 2048^2 launch (388 + 118 + 176 per node; the FP64 pipe 87 % busy). The
+# 2048^2 launch (230 + 79 + 117 per node; the FP64 pipe 88 % busy). The
 # FP64 kernel is bound by GB300's FP64 rate, not by HBM: its roofline is
 # reported against the nominal FP64 peak (there is no measured FP64 peak).
-FP64_FLOPS_PER_NODE = {"local": 1070.0}
+FP64_FLOPS_PER_NODE = {"local": 656.0}
 FP64_NOMINAL_TFLOPS = 1.25
 # Warp instructions per node-step of the FP32 step kernel with sampling every
 # step (tensor-core sums, 16 colliding warps), from ncu smsp__inst_executed.sum
-# of a 2048^2 launch (51.9 M and 53.7 M over 4.19 M nodes): with the issue rate
+# of a 2048^2 launch (51.6 M and 53.7 M over 4.19 M nodes): with the issue rate
 # of the GPU (4 schedulers per SM, one warp instruction per cycle each) they
 # give the issue ceiling the f-norm step is bound by.
-INSTR_PER_NODE = {("fp32", "local"): 12.37, ("fp32", "lut"): 12.80}
+INSTR_PER_NODE = {("fp32", "local"): 12.31, ("fp32", "lut"): 12.80}
 SCHEDULERS_PER_SM = 4
 
 
@@ -578,7 +578,7 @@ def bench_fp64(stream, p64, steps, peak, peak_kind):
     hbm = BYTES_PER_NODE["fp64"] * nodes / (ms * 1e-3) / 1e9
     out = {"workload": f"{p64.Lx}x{p64.Ly}, FP64 populations, the same parameters, sampled every step",
            "mlups": nodes / ms / 1e3, "ms_per_step": ms, "steps": steps,
-           "kernel": "step_kernel<f64,%s,sample>" % p64.basis,
+           "kernel": "step64_kernel<%s,sample>" % p64.basis,
            "hbm": {"achieved": hbm, "peak": peak, "unit": "GB/s", "frac": hbm / peak,
                    "peak_kind": peak_kind}}
     fl = FP64_FLOPS_PER_NODE.get(p64.basis)
@@ -654,7 +654,7 @@ def run_sweep(args, rank, world, dist, dev):
 def run_sweep21(args, rank, world, dist, dev):
     """--workload sweep21: the u_x0 sweep on the paper's own 21 x 21 lattice.
     --replicas independent copies per (u_x0, basis), all points of one basis in
-    one batch (one launch per step), --steps steps sampled every step after a
+    one batch (all steps of a call in one launch), --steps steps sampled every step after a
     tenth; the moment variances of the pooled copies (flb_batch_correlations)
     fitted as in the 4096^2 sweep, in the Hermite norm, the local f-norm and
     the table f-norm (the variant the paper's f-norm numbers come from)."""
@@ -904,7 +904,7 @@ def main():
     achieved = algo_bytes / (step_ms * 1e-3) / 1e9
     pipelined = args.precision == "fp32"
     kname = ("step_tma_kernel<%s,sample>" % args.basis) if pipelined else \
-        ("step_kernel<f64,%s,sample>" % args.basis)
+        ("step64_kernel<%s,sample>" % args.basis)
     traffic = DRAM_TRAFFIC.get((args.precision, args.basis, args.side))
     if args.pipeline_warps or args.pipeline_sampling or args.sample_every != 1:
         traffic = None
