@@ -3,6 +3,7 @@
 // grid sizing of the plain element-wise kernels and error-code mapping.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -15,32 +16,49 @@
 
 namespace flb {
 
-// Raise a kernel's dynamic shared memory limit on the current device to `bytes`,
+// The current context's number, unique for the life of the program: what is set
+// once per context is set again after a reset of the device. 0: unknown.
+inline unsigned long long context_id() {
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static const GetId get = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<GetId>(p);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+// Raise a kernel's dynamic shared memory limit in the current context to `bytes`,
 // unless an earlier call has: creating a lattice asked the runtime two dozen
 // times, about a third of the 230 us it took.
 inline cudaError_t allow_smem(const void* fn, size_t bytes) {
     struct Done {
-        int dev;
+        unsigned long long ctx;
         const void* fn;
         size_t bytes;
     };
     static std::mutex mutex;
     static std::vector<Done> done;
-    int dev = 0;
-    cudaError_t ce = cudaGetDevice(&dev);
-    if (ce != cudaSuccess) return ce;
+    const unsigned long long ctx = context_id();
+    if (!ctx) return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     std::lock_guard<std::mutex> lock(mutex);
     Done* mine = nullptr;
     for (Done& d : done)
-        if (d.dev == dev && d.fn == fn) mine = &d;
+        if (d.ctx == ctx && d.fn == fn) mine = &d;
     if (mine && mine->bytes >= bytes) return cudaSuccess;
-    ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const cudaError_t ce = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (ce != cudaSuccess) return ce;
     try {
         if (mine)
             mine->bytes = bytes;
         else
-            done.push_back({dev, fn, bytes});
+            done.push_back({ctx, fn, bytes});
     } catch (const std::bad_alloc&) {   // asked again next time
     }
     return cudaSuccess;

@@ -20,7 +20,10 @@
 
 #include <algorithm>
 #include <mutex>
+#include <new>
+#include <vector>
 
+#include "flb_host.h"
 #include "flb_step64.cuh"
 #include "flb_tma.cuh"
 
@@ -143,9 +146,12 @@ __global__ void __launch_bounds__(32) add_partials_kernel(const double* partials
     add_partials(partials, nblocks, acc, blockIdx.x);
 }
 
-constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
-NoiseTables g_tables[kMaxDevices];
+struct ContextTables {
+    unsigned long long ctx;
+    NoiseTables tables;
+};
+std::vector<ContextTables> g_tables;
 
 template <int BASIS, bool SAMPLE, bool SPLIT>
 cudaError_t launch(const Step64Args& a, const CollideConst<double>& cc, cudaStream_t s) {
@@ -166,39 +172,43 @@ cudaError_t launch(const Step64Args& a, const CollideConst<double>& cc, bool sam
 }  // namespace
 
 NoiseTables noise_tables() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+    const unsigned long long ctx = context_id();
+    if (!ctx) return NoiseTables();   // the kernel then forms the normals itself
+    std::lock_guard<std::mutex> lock(g_mutex);
+    for (const ContextTables& c : g_tables)
+        if (c.ctx == ctx) return c.tables;
+    NoiseTables t;
+    void* p = nullptr;
+    if (cudaMalloc(&p, sizeof(double) * kRadius + sizeof(double2) * kQuarter) != cudaSuccess) {
         cudaGetLastError();
         return NoiseTables();
     }
-    std::lock_guard<std::mutex> lock(g_mutex);
-    if (!g_tables[dev].radius) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, sizeof(double) * kRadius + sizeof(double2) * kQuarter) != cudaSuccess) {
-            cudaGetLastError();
-            return NoiseTables();
-        }
-        double2* circle = (double2*)p;
-        double* radius = (double*)(circle + kQuarter);
-        // on a stream of its own, then waited for (once per device)
-        cudaStream_t s;
-        cudaError_t ce = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-        if (ce == cudaSuccess) {
-            noise_tables_kernel<<<kRadius / 128, 128, 0, s>>>(radius, circle);
-            ce = cudaGetLastError();
-            const cudaError_t e2 = cudaStreamSynchronize(s);
-            if (ce == cudaSuccess) ce = e2;
-            cudaStreamDestroy(s);
-        }
-        if (ce != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(p);
-            return NoiseTables();
-        }
-        g_tables[dev].radius = radius;
-        g_tables[dev].circle = circle;
+    double2* circle = (double2*)p;
+    double* radius = (double*)(circle + kQuarter);
+    // on a stream of its own, then waited for (once per context)
+    cudaStream_t s;
+    cudaError_t ce = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (ce == cudaSuccess) {
+        noise_tables_kernel<<<kRadius / 128, 128, 0, s>>>(radius, circle);
+        ce = cudaGetLastError();
+        const cudaError_t e2 = cudaStreamSynchronize(s);
+        if (ce == cudaSuccess) ce = e2;
+        cudaStreamDestroy(s);
     }
-    return g_tables[dev];
+    if (ce != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(p);
+        return NoiseTables();
+    }
+    t.radius = radius;
+    t.circle = circle;
+    try {
+        g_tables.push_back({ctx, t});
+    } catch (const std::bad_alloc&) {
+        cudaFree(p);
+        return NoiseTables();
+    }
+    return t;
 }
 
 // About 16 blocks per SM, each with the same number of nodes per lane; fewer
