@@ -34,6 +34,9 @@ const void* kernel_of(int basis, bool half, bool sample) {
 // 7.1; 626 x 62 in 1 x 62 4.7, 2 x 62 4.4, 2 x 31 5.5, 7 x 21 7.3; 4000 x 20 in 2 / 4 / 7
 // x 20 10.5 / 5.7 / 5.0; 512 x 512 in 128 blocks 7.0, 2 x 74 7.1; 1000 x 750 in 150
 // 16.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
+// (Taken before the cells' byte addresses and the edges' scalar arguments, which
+// made a step 3 to 9 % faster: 21 x 21 sampled 2.0, 300 x 130 sampled 4.0, 1000 x 750
+// 15.0. The order of the cuts does not depend on that.)
 }  // namespace
 
 double resident_step_us(int wp, int gx, int gy, int bw, int bh) {
