@@ -24,6 +24,8 @@ const void* kernel_of(int basis, bool half, bool sample) {
     return half ? kernel_of<LatticePar16>(basis, sample) : kernel_of<LatticePar>(basis, sample);
 }
 
+}  // namespace
+
 // Estimated microseconds of a step (f-norm, no sampling): wp warp passes of 64
 // nodes on the four schedulers of an SM; blocks that exchange add their words'
 // trip through L2 and the passes whose lanes move them (a row on the edge; a
@@ -36,9 +38,7 @@ const void* kernel_of(int basis, bool half, bool sample) {
 // 16.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
 // (Taken before the cells' byte addresses and the edges' scalar arguments, which
 // made a step 3 to 9 % faster: 21 x 21 sampled 2.0, 300 x 130 sampled 4.0, 1000 x 750
-// 15.0. The order of the cuts does not depend on that.)
-}  // namespace
-
+// 15.0; the other cuts were not timed again.)
 double resident_step_us(int wp, int gx, int gy, int bw, int bh) {
     double t = std::max(1.75, 0.69 * ((wp + 3) / 4) + 0.3);
     if (gy > 1) t += 0.3 + 0.072 * bw / 32.0 + (bh == 1 ? 1.2 : 0.0);   // one row: two waits in a row
