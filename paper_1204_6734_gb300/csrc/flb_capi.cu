@@ -925,11 +925,10 @@ int flb_step(flb_lattice h, int64_t n) {
         int64_t run = n - s;
         float* const many = h->sk_every > 0 && uses_tma(h) ? structure_fields(h->sk) : nullptr;
         if (h->sk_every > 0) {
-            const int64_t next = h->t < h->sk_warmup ? h->sk_warmup
-                                                     : h->t + h->sk_every - (h->t - h->sk_warmup) % h->sk_every;
+            const int64_t next = h->t < h->sk_warmup ? h->sk_warmup - h->t
+                                                     : h->sk_every - (h->t - h->sk_warmup) % h->sk_every;
             const int64_t more = many ? structure_room(h->sk) - (sk_due ? 1 : 0) : 0;
-            run = next - h->t > run || h->sk_every > run ? std::min(run, next - h->t)
-                                                         : std::min(run, next - h->t + more * h->sk_every);
+            run = next > run || h->sk_every > run ? std::min(run, next) : std::min(run, next + more * h->sk_every);
         }
         run = ce == cudaSuccess ? resident_steps(h, run) : 0;
         if (run > 0) {

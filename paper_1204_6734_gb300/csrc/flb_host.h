@@ -124,14 +124,14 @@ inline bool tensor_sampling_ok(const flb_params* p) {
 }
 inline double gram_scale(const flb_params* p) { return std::sqrt(p->kT * p->rho0); }
 
-// Steps of [ta, tb) that the schedule (warmup, every) samples.
+// Steps of [ta, tb) that the schedule (warmup, every) samples. No sum of times
+// passes tb or warmup, so any `every` up to 2^63 - 1 will do.
 inline int64_t count_sampled(int64_t ta, int64_t tb, int64_t warmup, int64_t every) {
     if (every <= 0) return 0;
     const int64_t lo = ta > warmup ? ta : warmup;
     if (lo >= tb) return 0;
-    const int64_t first = warmup + (lo - warmup + every - 1) / every * every;
-    if (first >= tb) return 0;
-    return (tb - 1 - first) / every + 1;
+    const int64_t past = (lo - warmup) % every, skip = past ? every - past : 0;
+    return skip < tb - lo ? (tb - 1 - lo - skip) / every + 1 : 0;
 }
 
 // The device address of page-locked host memory, or null for other memory:
