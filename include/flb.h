@@ -345,6 +345,20 @@ int flb_batch_set_sampling(flb_batch b, int32_t slot, int64_t warmup, int64_t ev
  * Errors: FLB_ERR_ARG, FLB_ERR_CUDA. Device errors surface in sync/status. */
 int flb_batch_step(flb_batch b, int64_t n);
 
+/* Tuning and testing: FLB_KERNEL_AUTO (default) or FLB_KERNEL_PIPELINED (one
+ * launch per step, whatever the replicas' sizes). Errors: FLB_ERR_ARG. */
+int flb_batch_set_kernel(flb_batch b, int32_t kernel);
+
+/* What the last flb_batch_step (flb_step of a lattice) that took a step used:
+ * *kinds receives FLB_LAUNCH_* flags, *launches the number of step kernels
+ * (those in replayed graphs included). Either pointer may be NULL. */
+#define FLB_LAUNCH_STEP 1      /* one launch per step */
+#define FLB_LAUNCH_GRAPH 2     /* the same, replayed from a graph */
+#define FLB_LAUNCH_RESIDENT 4  /* many steps per launch, lattices whole */
+#define FLB_LAUNCH_CUT 8       /* many steps per launch, lattices in parts */
+int flb_batch_launches(flb_batch b, int32_t* kinds, int64_t* launches);
+int flb_launches(flb_lattice h, int32_t* kinds, int64_t* launches);
+
 /* Capture chunks of `steps` launches into a CUDA graph, replayed by
  * flb_batch_step (0 = launch every step directly; at most 100000). The graph
  * stays valid across membership changes. Must not be called while the

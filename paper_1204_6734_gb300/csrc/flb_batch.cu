@@ -80,6 +80,9 @@ struct flb_batch_s {
     size_t rsmem = 0;              // 0: one launch per step
     bool rcut = false;
     bool tune = false;             // the autotuner times the tile shapes
+    bool one_step = false;         // flb_batch_set_kernel
+    int kinds = 0;                 // FLB_LAUNCH_* of the last call, and its
+    int64_t launches = 0;          // step kernels
     uint32_t tag = 0;
     int graph_steps = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};   // [sample]
@@ -232,7 +235,7 @@ void plan_resident(flb_batch_s* b, bool sample) {
     b->rplan_dirty = false;
     b->rplan_sample = sample;
     b->rsmem = 0;
-    if (b->tune || (sample && !tensor_ok(b))) return;
+    if (sample && !tensor_ok(b)) return;
     const int mode = !sample ? kResQuiet : kBatchVariants[b->tile].tensor() ? kResStaged : kResExact;
     struct Item {
         int slot;
@@ -345,7 +348,7 @@ void plan_resident(flb_batch_s* b, bool sample) {
 // One launch of n steps; *done tells whether it was made.
 cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
     *done = false;
-    if (n < kResMinSteps || n > kResMaxSteps) return cudaSuccess;
+    if (b->tune || b->one_step || n < kResMinSteps || n > kResMaxSteps) return cudaSuccess;
     cudaError_t ce = cudaSuccess;
     if (b->rplan_dirty || b->rplan_sample != sample) {
         plan_resident(b, sample);
@@ -379,6 +382,8 @@ cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
     }
     if (ce != cudaSuccess) return ce;
     b->tag += (uint32_t)n;
+    b->kinds |= b->rcut ? FLB_LAUNCH_CUT : FLB_LAUNCH_RESIDENT;
+    b->launches += 1;
     *done = true;
     return ce;
 }
@@ -719,6 +724,8 @@ int flb_batch_step(flb_batch b, int64_t n) {
     bool sample = false;
     for (const BatchSlot& s : b->slots)
         if (s.used && s.every > 0 && b->step - s.join < s.tend) sample = true;
+    b->kinds = 0;
+    b->launches = 0;
     bool resident = false;
     cudaError_t ce = step_resident(b, sample, n, &resident);
     int64_t done = resident ? n : 0;
@@ -742,9 +749,15 @@ int flb_batch_step(flb_batch b, int64_t n) {
         while (ce == cudaSuccess && n - done >= b->graph_steps) {
             ce = cudaGraphLaunch(ge, b->stream);
             done += b->graph_steps;
+            b->kinds |= FLB_LAUNCH_GRAPH;
+            b->launches += b->graph_steps;
         }
     }
-    for (; done < n && ce == cudaSuccess; ++done) ce = launch(b, sample, b->stream);
+    for (; done < n && ce == cudaSuccess; ++done) {
+        ce = launch(b, sample, b->stream);
+        b->kinds |= FLB_LAUNCH_STEP;
+        b->launches += 1;
+    }
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_CUDA;
@@ -759,11 +772,24 @@ int flb_batch_step(flb_batch b, int64_t n) {
     return FLB_OK;
 }
 
+int flb_batch_set_kernel(flb_batch b, int32_t kernel) {
+    if (!b || (kernel != FLB_KERNEL_AUTO && kernel != FLB_KERNEL_PIPELINED)) return FLB_ERR_ARG;
+    b->one_step = kernel == FLB_KERNEL_PIPELINED;
+    return FLB_OK;
+}
+
+int flb_batch_launches(flb_batch b, int32_t* kinds, int64_t* launches) {
+    if (!b) return FLB_ERR_ARG;
+    if (kinds) *kinds = b->kinds;
+    if (launches) *launches = b->launches;
+    return FLB_OK;
+}
+
 int flb_batch_autotune(flb_batch b, int32_t trial_steps, int32_t* tile, double* ms_per_step) {
     if (!b || trial_steps < 1 || trial_steps > 100000) return FLB_ERR_ARG;
     const int keep_graph = b->graph_steps;
     b->graph_steps = 0;
-    b->tune = b->rplan_dirty = true;   // the tile shapes themselves, one launch per step
+    b->tune = true;   // the tile shapes themselves, one launch per step
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t ce = cudaEventCreate(&e0);
     if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
@@ -794,7 +820,6 @@ int flb_batch_autotune(flb_batch b, int32_t trial_steps, int32_t* tile, double* 
     if (e1) cudaEventDestroy(e1);
     b->graph_steps = keep_graph;
     b->tune = false;
-    b->rplan_dirty = true;
     if (ce != cudaSuccess) {
         cudaGetLastError();
         return FLB_ERR_CUDA;

@@ -346,6 +346,8 @@ struct flb_lattice_s {
     uint64_t* mail = nullptr;        // the blocks' mailboxes (two), when the lattice is cut
     uint32_t tag = 0;                // steps that resident launches made so far
     bool one_step = false;           // an option chose the one-step kernel's shape
+    int kinds = 0;                   // FLB_LAUNCH_* of the last flb_step, and its
+    int64_t launches = 0;            // step kernels
     const float* lut32 = nullptr;    // velocity tables (look-up-table f-norm)
     const double* lut64 = nullptr;
     double ref[9];
@@ -562,6 +564,8 @@ cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
     const cudaError_t ce = resident_step(h->res, a, collide_const<float>(&h->p), h->p.basis, half, ns > 0, h->stream);
     if (ce == cudaSuccess) {
         h->tag += (uint32_t)n;
+        h->kinds |= h->res.gx * h->res.gy > 1 ? FLB_LAUNCH_CUT : FLB_LAUNCH_RESIDENT;
+        h->launches += 1;
         h->nsamp += ns * (int64_t)h->p.Lx * h->p.Ly;
         h->t += n;
         h->cur ^= n & 1;
@@ -907,6 +911,10 @@ int flb_step(flb_lattice h, int64_t n) {
     if (!h || n < 0) return FLB_ERR_ARG;
     if (h->sticky) return h->sticky;
     const long long N = (long long)h->p.Lx * h->p.Ly;
+    if (n > 0) {
+        h->kinds = 0;
+        h->launches = 0;
+    }
     for (int64_t s = 0; s < n;) {
         const bool sample =
             h->every > 0 && h->t >= h->warmup && ((h->t - h->warmup) % h->every) == 0;
@@ -946,6 +954,8 @@ int flb_step(flb_lattice h, int64_t n) {
             ce = cudaSuccess;
         }
         if (ce == cudaSuccess) ce = launch_step(h, sample, fields);
+        h->kinds |= FLB_LAUNCH_STEP;
+        h->launches += 1;
         if (ce == cudaSuccess && fields) ce = structure_sample_fields(h->sk, 1, h->stream);
         if (ce == cudaSuccess && sample && !reduces_in_kernel(h)) {
             accumulate_partials_kernel<<<kSums, 32, 0, h->stream>>>(h->partials, h->nblocks,
@@ -962,6 +972,13 @@ int flb_step(flb_lattice h, int64_t n) {
         ++s;
     }
     if (flush64(h) != cudaSuccess) return FLB_ERR_CUDA;
+    return FLB_OK;
+}
+
+int flb_launches(flb_lattice h, int32_t* kinds, int64_t* launches) {
+    if (!h) return FLB_ERR_ARG;
+    if (kinds) *kinds = h->kinds;
+    if (launches) *launches = h->launches;
     return FLB_OK;
 }
 

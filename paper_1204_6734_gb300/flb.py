@@ -25,6 +25,7 @@ ERR_ARG, ERR_OOM, ERR_INVALID_VELOCITY, ERR_NONFINITE, ERR_TIMEOUT, ERR_CUDA, ER
 BASIS = {"standard": 0, "local": 1, "lut": 2}
 OPT_KERNEL, OPT_PIPELINE_WARPS, OPT_PIPELINE_SAMPLING = 0, 1, 2
 KERNEL = {"auto": 0, "generic": 1, "pipelined": 2}
+LAUNCH = {"step": 1, "graph": 2, "resident": 4, "cut": 8}   # kinds of launches of a call
 PRECISION = {"fp64": 0, "fp32": 1, "fp16dev": 2}
 TILE = {"128x4": 0, "64x8": 1, "128x2": 2, "128x6": 3, "64x12": 4, "mixed": 5}   # tile shapes of the batched kernel
 TILE_COUNT = 6
@@ -127,6 +128,9 @@ def load(build_if_missing: bool = True):
         "flb_batch_destroy": (C.c_int, [h]),
         "flb_batch_set_sampling": (C.c_int, [h, C.c_int32, C.c_int64, C.c_int64]),
         "flb_batch_step": (C.c_int, [h, C.c_int64]),
+        "flb_batch_set_kernel": (C.c_int, [h, C.c_int32]),
+        "flb_batch_launches": (C.c_int, [h, _i32p, _i64p]),
+        "flb_launches": (C.c_int, [h, _i32p, _i64p]),
         "flb_batch_set_graph": (C.c_int, [h, C.c_int32]),
         "flb_batch_set_tile": (C.c_int, [h, C.c_int32]),
         "flb_batch_get_tile": (C.c_int, [h, _i32p]),
@@ -170,6 +174,7 @@ def exported_symbols():
             "flb_version", "flb_state_difference", "flb_batch_open", "flb_batch_replica_bytes", "flb_batch_add",
             "flb_batch_remove", "flb_batch_create", "flb_batch_workspace_bytes",
             "flb_batch_destroy", "flb_batch_set_sampling", "flb_batch_step",
+            "flb_batch_set_kernel", "flb_batch_launches", "flb_launches",
             "flb_batch_set_graph", "flb_batch_set_tile", "flb_batch_get_tile",
             "flb_batch_autotune", "flb_batch_sync", "flb_batch_status", "flb_batch_time",
             "flb_batch_replica_time", "flb_batch_info", "flb_batch_raw_sums",
@@ -482,6 +487,27 @@ def flb_batch_step(b, n: int) -> None:
     _check(load().flb_batch_step(b, int(n)), "flb_batch_step")
 
 
+def flb_batch_set_kernel(b, kernel) -> None:
+    v = KERNEL[kernel] if isinstance(kernel, str) else int(kernel)
+    _check(load().flb_batch_set_kernel(b, v), "flb_batch_set_kernel")
+
+
+def _launches(name, h):
+    kinds, n = C.c_int32(), C.c_int64()
+    _check(getattr(load(), name)(h, C.byref(kinds), C.byref(n)), name)
+    return {k for k, bit in LAUNCH.items() if kinds.value & bit}, n.value
+
+
+def flb_batch_launches(b):
+    """The kinds of launches (keys of LAUNCH) of the last flb_batch_step and their number."""
+    return _launches("flb_batch_launches", b)
+
+
+def flb_launches(h):
+    """The kinds of launches (keys of LAUNCH) of the last flb_step and their number."""
+    return _launches("flb_launches", h)
+
+
 def flb_batch_set_graph(b, steps: int) -> None:
     _check(load().flb_batch_set_graph(b, int(steps)), "flb_batch_set_graph")
 
@@ -668,6 +694,9 @@ class Lattice:
     def t(self):
         return flb_time(self.h)
 
+    def launches(self):
+        return flb_launches(self.h)
+
     def populations(self):
         return flb_get_populations(self.h, self.p.Lx, self.p.Ly)
 
@@ -710,7 +739,7 @@ class Batch:
     limit; ``Batch.open(basis, max_replicas, pool_bytes)`` starts empty, for
     replicas that join and leave (``add`` / ``remove``)."""
 
-    def __init__(self, ps=None, stream=None, graph_steps=0, tile=None, _handle=None):
+    def __init__(self, ps=None, stream=None, graph_steps=0, tile=None, kernel=None, _handle=None):
         self.params = {}
         if _handle is not None:
             self.h = _handle
@@ -721,6 +750,8 @@ class Batch:
             flb_batch_set_graph(self.h, graph_steps)
         if tile is not None:
             flb_batch_set_tile(self.h, tile)
+        if kernel is not None:
+            flb_batch_set_kernel(self.h, kernel)
 
     @classmethod
     def open(cls, basis, max_replicas, pool_bytes, stream=None, graph_steps=0):
@@ -775,6 +806,12 @@ class Batch:
 
     def autotune(self, trial_steps=20):
         return flb_batch_autotune(self.h, trial_steps)
+
+    def set_kernel(self, kernel):
+        flb_batch_set_kernel(self.h, kernel)
+
+    def launches(self):
+        return flb_batch_launches(self.h)
 
     def set_graph(self, steps):
         flb_batch_set_graph(self.h, steps)
