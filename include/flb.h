@@ -341,7 +341,9 @@ int flb_batch_set_sampling(flb_batch b, int32_t slot, int64_t warmup, int64_t ev
  * advances by one time step in each. Batches whose replicas fit the SMs' shared
  * memory (small ones whole, a few larger ones in parts) make calls of three
  * steps or more in one launch; others take one launch per step, and with graphs
- * on (flb_batch_set_graph) whole chunks of them from a captured CUDA graph.
+ * on (flb_batch_set_graph) whole chunks of them from a captured CUDA graph. On a
+ * stream that the caller captures it is one launch per step; launch such a graph
+ * once, in the order of the calls, and before replicas join or leave.
  * Errors: FLB_ERR_ARG, FLB_ERR_CUDA. Device errors surface in sync/status. */
 int flb_batch_step(flb_batch b, int64_t n);
 

@@ -45,6 +45,14 @@ struct BatchSlot {
     float* buf[2] = {nullptr, nullptr};
 };
 
+// A replica in the plan of the resident launch.
+struct ResItem {
+    int slot;
+    int64_t nodes;
+    int g;        // blocks
+    double us;    // estimated time of its step
+};
+
 }  // namespace
 
 struct flb_batch_s {
@@ -63,7 +71,10 @@ struct flb_batch_s {
     double* scratch = nullptr;     // finalised correlations
     std::vector<BatchSlot> slots;
     std::vector<ReplicaDesc> hdesc;
+    // host sides of the tables, reserved at open: a captured copy of them reads
+    // them when the graph is launched, so they neither move nor end before the batch
     std::vector<uint32_t> htiles;
+    int hntiles = 0;
     int tile = 0;                  // FLB_TILE_*
     int grid = 1, sms = 1;
     int64_t step = 0;              // launches enqueued
@@ -74,6 +85,7 @@ struct flb_batch_s {
     uint64_t* mail = nullptr;      // mailboxes of cut replicas
     size_t mail_words = 0;         // words there is room for
     std::vector<ResCta> hrtable;
+    std::vector<ResItem> ritems;
     bool rplan_dirty = true;
     bool rplan_sample = false;
     int rmode = 0, rthreads = 0;
@@ -191,26 +203,37 @@ cudaError_t upload_desc(flb_batch_s* b, int slot) {
                            cudaMemcpyHostToDevice, b->stream);
 }
 
+// Whether the stream is being captured by the caller (or cannot be asked).
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // Rebuild the tile table from the live replicas (slot order) and upload it
-// with the tile count; takes effect at the next launch.
-cudaError_t upload_table(flb_batch_s* b) {
+// with the tile count; takes effect at the next launch. A captured upload is
+// part of the graph and has not run: the next call uploads again.
+cudaError_t upload_table(flb_batch_s* b, bool captured) {
     if (!b->table_dirty) return cudaSuccess;
     b->htiles.clear();
     for (int k = 0; k < b->cap; ++k) {
         const BatchSlot& s = b->slots[k];
         if (!s.used) continue;
         const int n = (int)replica_tiles(s.p, b->tile);
+        if (b->htiles.size() + n > b->max_tiles) return cudaErrorInvalidValue;
         for (int t = 0; t < n; ++t) b->htiles.push_back(((uint32_t)k << kLocalBits) | (uint32_t)t);
     }
-    if (b->htiles.size() > b->max_tiles) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     if (!b->htiles.empty())
         e = cudaMemcpyAsync(b->tiles, b->htiles.data(), sizeof(uint32_t) * b->htiles.size(),
                             cudaMemcpyHostToDevice, b->stream);
-    const int n = (int)b->htiles.size();
+    b->hntiles = (int)b->htiles.size();
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&b->ctl->ntiles, &n, sizeof(int), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) b->table_dirty = false;
+        e = cudaMemcpyAsync(&b->ctl->ntiles, &b->hntiles, sizeof(int), cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) b->table_dirty = captured;
     return e;
 }
 
@@ -237,13 +260,9 @@ void plan_resident(flb_batch_s* b, bool sample) {
     b->rsmem = 0;
     if (sample && !tensor_ok(b)) return;
     const int mode = !sample ? kResQuiet : kBatchVariants[b->tile].tensor() ? kResStaged : kResExact;
-    struct Item {
-        int slot;
-        int64_t nodes;
-        int g;
-        double us;
-    };
-    std::vector<Item> v;
+    using Item = ResItem;
+    std::vector<Item>& v = b->ritems;
+    v.clear();
     double padded = 0;
     for (int k = 0; k < b->cap; ++k) {
         const BatchSlot& s = b->slots[k];
@@ -345,7 +364,9 @@ void plan_resident(flb_batch_s* b, bool sample) {
     b->rmode = mode;
 }
 
-// One launch of n steps; *done tells whether it was made.
+// One launch of n steps; *done tells whether it was made. Not for a stream that is
+// being captured: the plan's upload would not have run when the next call relies
+// on it, and a mailbox tag may not be replayed.
 cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
     *done = false;
     if (b->tune || b->one_step || n < kResMinSteps || n > kResMaxSteps) return cudaSuccess;
@@ -361,14 +382,6 @@ cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
         }
     }
     if (!b->rsmem) return cudaSuccess;
-    if (b->rcut) {   // a mailbox tag may not be replayed
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(b->stream, &cap) != cudaSuccess) {
-            cudaGetLastError();
-            return cudaSuccess;
-        }
-        if (cap != cudaStreamCaptureStatusNone) return cudaSuccess;
-    }
     ResidentBatchArgs a{b->desc, b->rtable, b->ctl, b->lut, b->mail, b->tag, (int)n};
     void* params[1] = {(void*)&a};
     const void* fn = resident_batch_kernel_for(b->basis, b->rmode);
@@ -459,9 +472,6 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     b->basis = basis;
     b->cap = max_replicas;
     b->stream = (cudaStream_t)stream;
-    b->slots.resize(max_replicas);
-    b->hdesc.resize(max_replicas);
-    std::memset((void*)b->hdesc.data(), 0, sizeof(ReplicaDesc) * b->hdesc.size());
     // a replica of B pool bytes has at most B / 9216 tiles of 128 x 2 nodes
     b->max_tiles = pool_bytes / 9216 + (size_t)max_replicas;
     const size_t desc_bytes = Arena::round_up(sizeof(ReplicaDesc) * max_replicas);
@@ -477,6 +487,17 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
         delete b;
         return FLB_ERR_CUDA;
     }
+    try {   // all that later calls fill, so that they allocate no host memory
+        b->slots.resize(max_replicas);
+        b->hdesc.resize(max_replicas);
+        b->htiles.reserve(b->max_tiles);
+        b->hrtable.reserve(std::max(max_replicas, b->sms));
+        b->ritems.reserve(max_replicas);
+    } catch (const std::bad_alloc&) {
+        delete b;
+        return FLB_ERR_OOM;
+    }
+    std::memset((void*)b->hdesc.data(), 0, sizeof(ReplicaDesc) * b->hdesc.size());
     // the resident kernel's CTAs, and mailboxes for replicas it cuts (a row of
     // blocks exchanges 96 bytes per column, a node is 72 bytes of the pool)
     const size_t rtab_bytes = Arena::round_up(sizeof(ResCta) * std::max(max_replicas, b->sms));
@@ -726,10 +747,11 @@ int flb_batch_step(flb_batch b, int64_t n) {
         if (s.used && s.every > 0 && b->step - s.join < s.tend) sample = true;
     b->kinds = 0;
     b->launches = 0;
+    const bool captured = capturing(b->stream);
     bool resident = false;
-    cudaError_t ce = step_resident(b, sample, n, &resident);
+    cudaError_t ce = captured ? cudaSuccess : step_resident(b, sample, n, &resident);
     int64_t done = resident ? n : 0;
-    if (ce == cudaSuccess && !resident) ce = upload_table(b);
+    if (ce == cudaSuccess && !resident) ce = upload_table(b, captured);
     if (ce == cudaSuccess && b->graph_steps > 0 && n - done >= b->graph_steps) {
         cudaGraphExec_t& ge = b->graph[sample ? 1 : 0];
         if (!ge) {
