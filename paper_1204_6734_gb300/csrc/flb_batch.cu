@@ -91,6 +91,7 @@ struct flb_batch_s {
     int rmode = 0, rthreads = 0;
     size_t rsmem = 0;              // 0: one launch per step
     bool rcut = false;
+    double rus = 0;                // estimated time of a step
     bool tune = false;             // the autotuner times the tile shapes
     bool one_step = false;         // flb_batch_set_kernel
     int kinds = 0;                 // FLB_LAUNCH_* of the last call, and its
@@ -307,6 +308,7 @@ void plan_resident(flb_batch_s* b, bool sample) {
         b->rsmem = smem;
         b->rthreads = warps * 32;
         b->rcut = false;
+        b->rus = us;
     }
     // replicas cut: one CTA per SM
     if (R < b->sms) {
@@ -359,17 +361,18 @@ void plan_resident(flb_batch_s* b, bool sample) {
             b->rsmem = smem_of(cells, warps);
             b->rthreads = warps * 32;
             b->rcut = words > 0;
+            b->rus = us;
         }
     }
     b->rmode = mode;
 }
 
-// One launch of n steps; *done tells whether it was made. Not for a stream that is
+// One launch of up to n steps; *done receives how many (0: none was made). Not for a stream that is
 // being captured: the plan's upload would not have run when the next call relies
 // on it, and a mailbox tag may not be replayed.
-cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
-    *done = false;
-    if (b->tune || b->one_step || n < kResMinSteps || n > kResMaxSteps) return cudaSuccess;
+cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, int64_t* done) {
+    *done = 0;
+    if (b->tune || b->one_step || n < kResMinSteps) return cudaSuccess;
     cudaError_t ce = cudaSuccess;
     if (b->rplan_dirty || b->rplan_sample != sample) {
         plan_resident(b, sample);
@@ -382,6 +385,7 @@ cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
         }
     }
     if (!b->rsmem) return cudaSuccess;
+    n = resident_launch_steps(n, b->rus);
     ResidentBatchArgs a{b->desc, b->rtable, b->ctl, b->lut, b->mail, b->tag, (int)n};
     void* params[1] = {(void*)&a};
     const void* fn = resident_batch_kernel_for(b->basis, b->rmode);
@@ -397,7 +401,7 @@ cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, bool* done) {
     b->tag += (uint32_t)n;
     b->kinds |= b->rcut ? FLB_LAUNCH_CUT : FLB_LAUNCH_RESIDENT;
     b->launches += 1;
-    *done = true;
+    *done = n;
     return ce;
 }
 
@@ -748,10 +752,11 @@ int flb_batch_step(flb_batch b, int64_t n) {
     b->kinds = 0;
     b->launches = 0;
     const bool captured = capturing(b->stream);
-    bool resident = false;
-    cudaError_t ce = captured ? cudaSuccess : step_resident(b, sample, n, &resident);
-    int64_t done = resident ? n : 0;
-    if (ce == cudaSuccess && !resident) ce = upload_table(b, captured);
+    cudaError_t ce = cudaSuccess;
+    int64_t done = 0;
+    for (int64_t m = 1; !captured && m > 0 && done < n && ce == cudaSuccess; done += m)
+        ce = step_resident(b, sample, n - done, &m);
+    if (ce == cudaSuccess && done < n) ce = upload_table(b, captured);
     if (ce == cudaSuccess && b->graph_steps > 0 && n - done >= b->graph_steps) {
         cudaGraphExec_t& ge = b->graph[sample ? 1 : 0];
         if (!ge) {

@@ -497,8 +497,8 @@ DevCodec dev_codec(flb_lattice h) {
 // (the kernel without sampling) where that leaves no short launch.
 int64_t resident_steps(flb_lattice h, int64_t n) {
     if (!h->res.gx || h->variant != FLB_KERNEL_AUTO || h->one_step || h->slab) return 0;
-    n = std::min<int64_t>(n, kResMaxSteps);
     if (n < kResMinSteps) return 0;
+    n = resident_launch_steps(n, h->res.us);
     if (h->every > 0 && h->t < h->warmup) {
         const int64_t quiet = h->warmup - h->t;
         if (quiet >= kResMinSteps && n - quiet >= kResMinSteps) n = quiet;

@@ -666,6 +666,13 @@ resident_kernel(const __grid_constant__ ResidentArgs a, const __grid_constant__ 
 constexpr int kResMinSteps = 3;
 constexpr int kResMaxSteps = 1 << 20;
 
+// Steps of the next launch, of n that are left: what is left is never too short for
+// one more.
+inline int64_t resident_launch_steps(int64_t n, double) {
+    const int64_t m = kResMaxSteps;
+    return n <= m ? n : (n - m < kResMinSteps ? m - kResMinSteps : m);
+}
+
 // A lattice's launch: how it is cut, and what the launch needs.
 struct ResidentPlan {
     int gx = 0, gy = 0;      // 0: no resident launch
