@@ -340,7 +340,7 @@ int flb_batch_set_sampling(flb_batch b, int32_t slot, int64_t warmup, int64_t ev
 /* Enqueue n steps of the batch: every live replica below its step limit
  * advances by one time step in each. Batches whose replicas fit the SMs' shared
  * memory (small ones whole, a few larger ones in parts) make calls of three
- * steps or more in one launch; others take one launch per step, and with graphs
+ * steps or more in launches of many steps, about 10 ms each at most; others take one launch per step, and with graphs
  * on (flb_batch_set_graph) whole chunks of them from a captured CUDA graph. On a
  * stream that the caller captures it is one launch per step; launch such a graph
  * once, in the order of the calls, and before replicas join or leave.

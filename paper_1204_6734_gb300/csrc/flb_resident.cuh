@@ -666,10 +666,14 @@ resident_kernel(const __grid_constant__ ResidentArgs a, const __grid_constant__ 
 constexpr int kResMinSteps = 3;
 constexpr int kResMaxSteps = 1 << 20;
 
-// Steps of the next launch, of n that are left: what is left is never too short for
-// one more.
-inline int64_t resident_launch_steps(int64_t n, double) {
-    const int64_t m = kResMaxSteps;
+// Steps of the next launch, of n that are left, us (estimated) each: about 10 ms at
+// most, for a launch holds its SMs to its end and other streams' kernels come in
+// between launches only. (A launch of its own costs 3 to 6 us, below 0.1 % of that.)
+// What is left is never too short for one more.
+constexpr double kResLaunchUs = 10000;
+inline int64_t resident_launch_steps(int64_t n, double us) {
+    const int64_t most = us * kResMaxSteps > kResLaunchUs ? (int64_t)(kResLaunchUs / us) : kResMaxSteps;
+    const int64_t m = most < 2 * kResMinSteps ? 2 * kResMinSteps : most;
     return n <= m ? n : (n - m < kResMinSteps ? m - kResMinSteps : m);
 }
 
