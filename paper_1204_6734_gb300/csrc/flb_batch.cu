@@ -249,7 +249,7 @@ int warp_passes(int64_t cells) { return (int)(((cells + 1) / 2 + 31) / 32); }
 // Plan the resident launch of the present members, or find that one launch per
 // step is faster (rsmem = 0). Small replicas as they are, several CTAs per SM;
 // or, with fewer replicas than SMs, the SMs dealt out one by one to the replica
-// whose step takes longest. Measured, us per step against one launch per step,
+// whose step takes longest, as far as the mailboxes have room. Measured, us per step against one launch per step,
 // f-norm, sampled with FP32 products: 384 x 21^2 6.1 against 61.5 (4.8 / 30.1
 // without sampling), 24 x 21^2 2.5 / 14.4, 1280 x 21^2 16.0 / 169, 300 x 48^2
 // 17.1 / 63.6, 8 x 64^2 (cut) 4.4 / 14.4; two to four CTAs per SM within 1 %. A
@@ -320,7 +320,12 @@ void plan_resident(flb_batch_s* b, bool sample) {
             const flb_params& p = b->slots[i.slot].p;
             return resident_step_us(warp_passes(cells_of(i, g)), 1, g, p.Lx, (p.Ly + g - 1) / g);
         };
+        const auto words_of = [&](const Item& i, int g) {
+            const flb_params& p = b->slots[i.slot].p;
+            return 2 * res_mail_words(p.Lx, p.Ly, 1, g);
+        };
         int used = 0;
+        long long mail = 0;
         bool ok = true;
         for (Item& i : v) {
             const int Ly = b->slots[i.slot].p.Ly;
@@ -328,16 +333,19 @@ void plan_resident(flb_batch_s* b, bool sample) {
             ok = ok && smem_of(cells_of(i, i.g), kResMaxWarps) <= kResSmemMax;
             i.us = us_of(i, i.g);
             used += i.g;
+            mail += words_of(i, i.g);
         }
-        ok = ok && used <= b->sms;
+        ok = ok && used <= b->sms && mail <= (long long)b->mail_words;
         while (ok && used < b->sms) {
             Item& i = *std::max_element(v.begin(), v.end(), [](const Item& a, const Item& c) { return a.us < c.us; });
             // the next cut that makes its blocks smaller
             const int Ly = b->slots[i.slot].p.Ly, rows = (Ly + i.g - 1) / i.g;
             if (rows <= 1) break;
             const int g = (Ly + rows - 2) / (rows - 1);
-            if (used + g - i.g > b->sms || us_of(i, g) >= i.us) break;
+            const long long more = words_of(i, g) - words_of(i, i.g);
+            if (used + g - i.g > b->sms || mail + more > (long long)b->mail_words || us_of(i, g) >= i.us) break;
             used += g - i.g;
+            mail += more;
             i.g = g;
             i.us = us_of(i, g);
         }
@@ -349,7 +357,7 @@ void plan_resident(flb_batch_s* b, bool sample) {
             words += res_mail_words(b->slots[i.slot].p.Lx, b->slots[i.slot].p.Ly, 1, i.g);
         }
         us *= sample ? 1.2 : 1.0;
-        if (ok && us < best && (size_t)(2 * words) <= b->mail_words) {
+        if (ok && us < best) {
             b->hrtable.clear();
             int at = 0;
             for (const Item& i : v) {
@@ -367,9 +375,9 @@ void plan_resident(flb_batch_s* b, bool sample) {
     b->rmode = mode;
 }
 
-// One launch of up to n steps; *done receives how many (0: none was made). Not for a stream that is
-// being captured: the plan's upload would not have run when the next call relies
-// on it, and a mailbox tag may not be replayed.
+// One launch of up to n steps; *done receives how many (0: none was made). Not for
+// a stream that is being captured: the plan's upload would not have run when the
+// next call relies on it, and a mailbox tag may not be replayed.
 cudaError_t step_resident(flb_batch_s* b, bool sample, int64_t n, int64_t* done) {
     *done = 0;
     if (b->tune || b->one_step || n < kResMinSteps) return cudaSuccess;
