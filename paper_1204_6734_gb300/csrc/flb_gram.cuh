@@ -165,72 +165,6 @@ __device__ __forceinline__ void gram_mma_rn(const GramLane& g, float (&c)[8]) {
     gram_step_rn<3>(g.ld, c);
 }
 
-// The same sums from deviations staged as two FP16 numbers, h + l with l the
-// rounding error of h rounded again: 22 bits of a value, so that the products
-// h h + h l + l h carry FP32's accuracy (l l, below 2^-22 of them, is left out).
-// The l block has the layout of the h block, its row 9 zero. Every 16 nodes
-// start from zero and are added to the sums outside the tensor cores, rounded to
-// nearest: their accumulators cut off instead, which biased the second moments
-// by 1e-6 when they ran over the 24 products of a block of 64 nodes.
-__device__ __forceinline__ void gram_zero_row(__half* blk) {
-    reinterpret_cast<uint32_t*>(blk)[9 * (kGramRowHalves / 2) + (threadIdx.x & 31)] = 0u;
-}
-
-template <int I>
-__device__ __forceinline__ void gram_store_pair(uint32_t st, uint32_t sl, f2 h) {
-    const __half2 v = __floats2half2_rn(h.v.x, h.v.y);
-    const float2 b = __half22float2(v);
-    const f2 d = h - f2(b);
-    const __half2 w = __floats2half2_rn(d.v.x, d.v.y);
-    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(st), "n"(2 * kGramRowHalves * I),
-                 "r"(*reinterpret_cast<const uint32_t*>(&v)));
-    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(sl), "n"(2 * kGramRowHalves * I),
-                 "r"(*reinterpret_cast<const uint32_t*>(&w)));
-}
-
-__device__ __forceinline__ void gram_stage_pair(const GramLane& g, const GramLane& l, const f2 (&h)[9]) {
-    __syncwarp();
-    gram_store_pair<0>(g.st, l.st, h[0]);
-    gram_store_pair<1>(g.st, l.st, h[1]);
-    gram_store_pair<2>(g.st, l.st, h[2]);
-    gram_store_pair<3>(g.st, l.st, h[3]);
-    gram_store_pair<4>(g.st, l.st, h[4]);
-    gram_store_pair<5>(g.st, l.st, h[5]);
-    gram_store_pair<6>(g.st, l.st, h[6]);
-    gram_store_pair<7>(g.st, l.st, h[7]);
-    gram_store_pair<8>(g.st, l.st, h[8]);
-}
-
-template <int S>
-__device__ __forceinline__ void gram_step_pair(uint32_t ld, uint32_t ll, float (&c)[8]) {
-    uint32_t d0, d1, d2, d3, e0, e1, e2, e3;
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4+%5];"
-                 : "=r"(d0), "=r"(d1), "=r"(d2), "=r"(d3)
-                 : "r"(ld), "n"(32 * S));
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4+%5];"
-                 : "=r"(e0), "=r"(e1), "=r"(e2), "=r"(e3)
-                 : "r"(ll), "n"(32 * S));
-    float p[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) p[q] = 0.f;
-    mma16816(p, 0, d0, d1, d2, d3, d0, d2);
-    mma16816(p, 4, d0, d1, d2, d3, d1, d3);
-    mma16816(p, 0, d0, d1, d2, d3, e0, e2);
-    mma16816(p, 4, d0, d1, d2, d3, e1, e3);
-    mma16816(p, 0, e0, e1, e2, e3, d0, d2);
-    mma16816(p, 4, e0, e1, e2, e3, d1, d3);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) c[q] += p[q];
-}
-
-__device__ __forceinline__ void gram_mma_pair(const GramLane& g, const GramLane& l, float (&c)[8]) {
-    __syncwarp();
-    gram_step_pair<0>(g.ld, l.ld, c);
-    gram_step_pair<1>(g.ld, l.ld, c);
-    gram_step_pair<2>(g.ld, l.ld, c);
-    gram_step_pair<3>(g.ld, l.ld, c);
-}
-
 // Add the FP32 partials to the FP64 matrix cm[16][16] (rows and columns 0..9
 // only) and clear them. Fragment of thread (g, q) = (lane / 4, lane % 4):
 // c[0..3] = C[g][2q], C[g][2q+1], C[g+8][2q], C[g+8][2q+1]; c[4..7] the same
@@ -257,6 +191,148 @@ __device__ __forceinline__ double gram_sum(const double* cm, int q, double s) {
         ++i;
     }
     return s * s * cm[i * 16 + i + k];
+}
+
+// ---------------------------------------------------------------------------
+// The same sums with FP32 products, rounded to nearest throughout: for batches in
+// the tile shapes that promise them.
+//
+// A warp stages its 64 nodes in FP32 (rows 0..8, row 9 ones). The ten rows make
+// five pairs, the upper triangle of their products 15 blocks of 2 x 2 entries, and
+// two lanes share a block, each with every other four nodes: 32 128-bit loads and
+// 64 packed multiply-adds per 64 nodes, four packed sums per lane across tiles.
+// Rows are 68 floats apart, so that the lanes of a load meet two banks twice at
+// most. Tensor cores cut off where this rounds: with deviations in two FP16 halves in
+// place of FP32 products <df df> was 2e-7 too small.
+// ---------------------------------------------------------------------------
+constexpr int kProdRowFloats = 68;                        // 64 nodes + 4 floats
+constexpr int kProdWarpFloats = 10 * kProdRowFloats;      // one warp's block: 2720 bytes
+constexpr int kProdBlocks = 15, kProdEntries = 4 * kProdBlocks;
+
+// Entry of rows i <= j (0..9) among a warp's kProdEntries sums.
+__host__ __device__ constexpr int prod_entry(int i, int j) {
+    const int p = i >> 1, q = j >> 1;
+    return 4 * (5 * p - p * (p - 1) / 2 + q - p) + 2 * (i & 1) + (j & 1);
+}
+static_assert(prod_entry(0, 0) == 0 && prod_entry(2, 2) == 20 && prod_entry(9, 9) == kProdEntries - 1, "15 blocks");
+
+// Shared addresses of one thread in its warp's block: the column pair it stages
+// and the first four values of the two row pairs it multiplies.
+struct ProdLane {
+    uint32_t st, a, b;
+    __device__ __forceinline__ explicit ProdLane(uint32_t blk) {
+        const int lane = threadIdx.x & 31, half = lane >= kProdBlocks && lane < 2 * kProdBlocks;
+        int p = 0, q = lane % kProdBlocks;   // lanes 30 and 31 repeat lanes 0 and 1
+        while (q >= 5 - p) {
+            q -= 5 - p;
+            ++p;
+        }
+        q += p;
+        st = blk + 8u * lane;
+        a = blk + 8u * kProdRowFloats * p + 16u * half;
+        b = blk + 8u * kProdRowFloats * q + 16u * half;
+    }
+};
+
+__device__ __forceinline__ void prod_init(float* blk) {
+    reinterpret_cast<float2*>(blk + 9 * kProdRowFloats)[threadIdx.x & 31] = make_float2(1.f, 1.f);
+}
+
+template <int I>
+__device__ __forceinline__ void prod_store(uint32_t st, f2 d) {
+    asm volatile("st.shared.v2.f32 [%0+%1], {%2,%3};" ::"r"(st), "n"(4 * kProdRowFloats * I), "f"(d.v.x), "f"(d.v.y));
+}
+
+// Stage the 64 nodes of this warp (d: node A of the thread in .x, node B in .y, zero
+// for nodes outside the lattice).
+__device__ __forceinline__ void prod_stage(const ProdLane& g, const f2 (&d)[9]) {
+    __syncwarp();
+    prod_store<0>(g.st, d[0]);
+    prod_store<1>(g.st, d[1]);
+    prod_store<2>(g.st, d[2]);
+    prod_store<3>(g.st, d[3]);
+    prod_store<4>(g.st, d[4]);
+    prod_store<5>(g.st, d[5]);
+    prod_store<6>(g.st, d[6]);
+    prod_store<7>(g.st, d[7]);
+    prod_store<8>(g.st, d[8]);
+}
+
+// Four nodes of the row at byte offset O.
+template <int O>
+__device__ __forceinline__ float4 prod_load(uint32_t p) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4+%5];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(p), "n"(O));
+    return v;
+}
+
+template <int E>
+__device__ __forceinline__ void prod_add(float (&c)[8], float4 x, float4 y) {
+    f2 v(c[2 * E], c[2 * E + 1]);
+    v = mad(f2(x.x, x.y), f2(y.x, y.y), v);
+    v = mad(f2(x.z, x.w), f2(y.z, y.w), v);
+    c[2 * E] = v.v.x;
+    c[2 * E + 1] = v.v.y;
+}
+
+template <int K>
+__device__ __forceinline__ void prod_step(const ProdLane& g, float (&c)[8]) {
+    const float4 a0 = prod_load<32 * K>(g.a), a1 = prod_load<32 * K + 4 * kProdRowFloats>(g.a);
+    const float4 b0 = prod_load<32 * K>(g.b), b1 = prod_load<32 * K + 4 * kProdRowFloats>(g.b);
+    prod_add<0>(c, a0, b0);
+    prod_add<1>(c, a0, b1);
+    prod_add<2>(c, a1, b0);
+    prod_add<3>(c, a1, b1);
+}
+
+// Add the products of the staged nodes to c.
+__device__ __forceinline__ void prod_sums(const ProdLane& g, float (&c)[8]) {
+    __syncwarp();
+    prod_step<0>(g, c);
+    prod_step<1>(g, c);
+    prod_step<2>(g, c);
+    prod_step<3>(g, c);
+    prod_step<4>(g, c);
+    prod_step<5>(g, c);
+    prod_step<6>(g, c);
+    prod_step<7>(g, c);
+}
+
+// The warp's sums of block `lane` (lanes below kProdBlocks); clears c.
+__device__ __forceinline__ float4 prod_take(float (&c)[8]) {
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        v[e] = c[2 * e] + c[2 * e + 1];
+        v[e] += __shfl_down_sync(0xffffffffu, v[e], kProdBlocks);
+        c[2 * e] = c[2 * e + 1] = 0.f;
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// Add the FP32 partials to kProdEntries FP64 sums in shared memory and clear them.
+__device__ __forceinline__ void prod_flush(float (&c)[8], double* sums) {
+    const int lane = threadIdx.x & 31;
+    const float4 v = prod_take(c);
+    if (lane < kProdBlocks) {
+        atomicAdd(&sums[4 * lane], (double)v.x);
+        atomicAdd(&sums[4 * lane + 1], (double)v.y);
+        atomicAdd(&sums[4 * lane + 2], (double)v.z);
+        atomicAdd(&sums[4 * lane + 3], (double)v.w);
+    }
+}
+
+// Sum q of the kSums layout, the staged values being d / s.
+__device__ __forceinline__ double prod_sum(const double* sums, int q, double s) {
+    if (q < 9) return s * sums[prod_entry(q, 9)];
+    int k = q - 9, i = 0;
+    while (k >= 9 - i) {
+        k -= 9 - i;
+        ++i;
+    }
+    return s * s * sums[prod_entry(i, i + k)];
 }
 
 }  // namespace flb

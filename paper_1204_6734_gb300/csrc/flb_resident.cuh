@@ -41,12 +41,10 @@
 // very nodes that read it, so no reader can be overtaken. All CTAs are
 // resident at once (cooperative launch), every wait is bounded (flb_tma.cuh).
 //
-// Correlation sums: as flb_gram.cuh, except that every step's FP32 partials
-// (at most 1024 products per warp, added over the CTA's warps in FP32 in a
-// fixed order) go to FP64 by themselves: the sums do not depend on how many
-// steps a launch makes. Where a batch's tile shape promises FP32 products, the
-// deviations are staged as two FP16 numbers (h + l, 22 bits) and the products
-// are h h + h l + l h, all exact in the FP32 accumulator's inputs.
+// Correlation sums: as flb_gram.cuh (staged in FP16 for the tensor cores, or with
+// FP32 products where a batch's tile shape promises them), except that every step's FP32 partials (at most 1024 products per warp, added
+// over the CTA's warps in FP32 in a fixed order) go to FP64 by themselves: the sums
+// do not depend on how many steps a launch makes.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -61,16 +59,17 @@
 namespace flb {
 
 constexpr int kResMaxWarps = 16;   // 512 threads of 128 registers
-constexpr int kResEntries = 84;    // Gram entries kept: rows 0..7 x columns 0..9, rows 8, 9 x 8, 9
 constexpr int kResSlot = 96;       // floats per warp and parity
 
 // Sampling of a resident launch: none; deviations staged in FP16; FP32 products.
 enum : int { kResQuiet = 0, kResStaged = 1, kResExact = 2 };
+// Entries kept: of the Gram matrix rows 0..7 x columns 0..9 and rows 8, 9 x 8, 9.
+__host__ __device__ constexpr int res_entries(int mode) { return mode == kResExact ? kProdEntries : 84; }
 
 __host__ __device__ constexpr size_t res_cells_bytes(int cells) { return ((size_t)cells * 36 + 15) / 16 * 16; }
 __host__ __device__ constexpr size_t res_sample_bytes(int mode, int warps) {
     return mode == kResQuiet ? 0
-                             : (size_t)warps * ((mode == kResExact ? 2 : 1) * kGramWarpHalves * 2 + 2 * kResSlot * 4) +
+                             : (size_t)warps * ((mode == kResExact ? kProdWarpFloats * 4 : kGramWarpHalves * 2) + 2 * kResSlot * 4) +
                                    kResSlot * 8;
 }
 // Dynamic shared memory of a CTA of `warps` warps holding `cells` nodes.
@@ -296,11 +295,17 @@ __device__ __forceinline__ void res_edge_out(uint64_t* out, uint32_t tag, const 
                                a.b<opposite(I0)>(), a.b<opposite(I1)>(), a.b<opposite(I2)>(), skip1, skip2, both);
 }
 
-// A warp's FP32 partials of one step, in the order of the kept entries (C is
-// symmetric): rows 0..7 by columns 0..7, rows 0..7 by columns 8 and 9, rows 8
+// A warp's FP32 partials of one step: with FP32 products in prod_entry's order, else
+// in the order of the kept entries (C is symmetric): rows 0..7 by columns 0..7, rows 0..7 by columns 8 and 9, rows 8
 // and 9 by columns 8 and 9. Cleared for the next sampled step.
+template <int SAMPLE>
 __device__ __forceinline__ void res_publish(float (&c)[8], float* slot) {
     const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    if constexpr (SAMPLE == kResExact) {
+        const float4 v = prod_take(c);
+        if (lane < kProdBlocks) *reinterpret_cast<float4*>(slot + 4 * lane) = v;
+        return;
+    }
     *reinterpret_cast<float2*>(slot + 2 * lane) = make_float2(c[0], c[1]);
     if (q == 0) {
         *reinterpret_cast<float2*>(slot + 64 + 2 * g) = make_float2(c[4], c[5]);
@@ -314,9 +319,10 @@ __device__ __forceinline__ void res_publish(float (&c)[8], float* slot) {
 // the last 96 threads of the CTA (warps without nodes of their own where the
 // block leaves room for them; entry q always by the same thread). All loads are
 // under way before the first add: this sits in the step's critical path.
+template <int SAMPLE>
 __device__ __forceinline__ void res_reduce(const float* slots, double* red, int nw) {
     const int T = blockDim.x, r0 = T > kResSlot ? T - kResSlot : 0;
-    for (int q = (int)threadIdx.x - r0; q >= 0 && q < kResEntries; q += T) {
+    for (int q = (int)threadIdx.x - r0; q >= 0 && q < res_entries(SAMPLE); q += T) {
         float v[kResMaxWarps];
 #pragma unroll
         for (int w = 0; w < kResMaxWarps; ++w) v[w] = w < nw ? slots[w * kResSlot + q] : 0.f;
@@ -329,7 +335,9 @@ __device__ __forceinline__ void res_reduce(const float* slots, double* red, int 
 }
 
 // Sum q of the kSums layout from the kept entries.
+template <int SAMPLE>
 __device__ __forceinline__ double res_sum(const double* red, int q, double s) {
+    if constexpr (SAMPLE == kResExact) return prod_sum(red, q, s);
     if (q < 9) return s * red[q < 8 ? 64 + 2 * q + 1 : 81];
     int k = q - 9, i = 0;
     while (k >= 9 - i) {
@@ -360,17 +368,19 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
         reinterpret_cast<volatile int*>(after + res_sample_bytes(SAMPLE, nw));
     if (c == 0) *gave_up = 0;
 
-    constexpr int kBlocks = SAMPLE == kResExact ? 2 : 1;
-    __half* blk = gram + warp * kBlocks * kGramWarpHalves;
-    const GramLane gh(SAMPLE ? smem_u32(blk) : 0u, kGramRows);
-    const GramLane gl(SAMPLE == kResExact ? smem_u32(blk + kGramWarpHalves) : 0u, kGramRows);
+    constexpr bool kExact = SAMPLE == kResExact;
+    const uint32_t blk = SAMPLE ? smem_u32(gram) + warp * (kExact ? kProdWarpFloats * 4 : kGramWarpHalves * 2) : 0u;
+    const GramLane gh(kExact ? 0u : blk, kGramRows);
+    const ProdLane gp(kExact ? blk : 0u);
     float gc[SAMPLE ? 8 : 1];
     if constexpr (SAMPLE != kResQuiet) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) gc[q] = 0.f;
-        gram_init(blk);
-        if constexpr (SAMPLE == kResExact) gram_zero_row(blk + kGramWarpHalves);
-        for (int q = c - (T > kResSlot ? T - kResSlot : 0); q >= 0 && q < kResEntries; q += T) red[q] = 0.0;
+        if constexpr (kExact)
+            prod_init(reinterpret_cast<float*>(gram) + warp * kProdWarpFloats);
+        else
+            gram_init(gram + warp * kGramWarpHalves);
+        for (int q = c - (T > kResSlot ? T - kResSlot : 0); q >= 0 && q < res_entries(SAMPLE); q += T) red[q] = 0.0;
     }
 
     // this thread's nodes: pairs c, c + T, ...
@@ -421,7 +431,7 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
         const bool smp = SAMPLE != kResQuiet && st == until;
         if (smp) until = k.every > k.n - st ? k.n : st + k.every;
         if constexpr (SAMPLE != kResQuiet) {
-            if (pending) res_reduce(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
+            if (pending) res_reduce<SAMPLE>(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
             pending = false;
         }
         float* fields = nullptr;
@@ -512,8 +522,8 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
                             h[i] = par.scaled(gg[i], i);
                             if (!inB) h[i] = f2(inA ? h[i].v.x : 0.f, 0.f);
                         }
-                        if constexpr (SAMPLE == kResExact)
-                            gram_stage_pair(gh, gl, h);
+                        if constexpr (kExact)
+                            prod_stage(gp, h);
                         else
                             gram_stage(gh, h);
                     }
@@ -551,8 +561,8 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
             // after the stores: what the neighbours wait for leaves first
             if constexpr (SAMPLE != kResQuiet) {
                 if (smp) {
-                    if constexpr (SAMPLE == kResExact)
-                        gram_mma_pair(gh, gl, reinterpret_cast<float(&)[8]>(gc));
+                    if constexpr (kExact)
+                        prod_sums(gp, reinterpret_cast<float(&)[8]>(gc));
                     else if constexpr (sizeof(Store) == 2)
                         gram_mma_rn(gh, reinterpret_cast<float(&)[8]>(gc));
                     else
@@ -571,7 +581,7 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
         if constexpr (SAMPLE != kResQuiet) {
             if (smp) {
                 if (warp < nwork)
-                    res_publish(reinterpret_cast<float(&)[8]>(gc), slots + ((nsum & 1) * nw + warp) * kResSlot);
+                    res_publish<SAMPLE>(reinterpret_cast<float(&)[8]>(gc), slots + ((nsum & 1) * nw + warp) * kResSlot);
                 ++nsum;
                 pending = true;
             }
@@ -582,10 +592,10 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
     }
     if constexpr (SAMPLE != kResQuiet) {
         __syncthreads();
-        if (pending) res_reduce(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
+        if (pending) res_reduce<SAMPLE>(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
         __syncthreads();
         if (nsum)
-            for (int q = c; q < kSums; q += T) atomicAdd(&k.acc[q], res_sum(red, q, par.s));
+            for (int q = c; q < kSums; q += T) atomicAdd(&k.acc[q], res_sum<SAMPLE>(red, q, par.s));
     }
 }
 

@@ -13,10 +13,9 @@ struct ReplicaPar {
     const CollidePairs& cc;
     const ReplicaHot& h;
     double s;
-    // with FP32 products the deviation itself first (an exact difference): the
-    // roundings of ref / s and 1 / s would bias the first moments
+    // with FP32 products the deviation itself
     __device__ __forceinline__ f2 scaled(f2 f, int i) const {
-        return SAMPLE == kResExact ? (f - f2(h.ref[i])) * f2(h.sinv) : mad(f, f2(h.sinv), f2(h.snref[i]));
+        return SAMPLE == kResExact ? f - f2(h.ref[i]) : mad(f, f2(h.sinv), f2(h.snref[i]));
     }
     __device__ __forceinline__ float ref(int i) const { return h.ref[i]; }
     __device__ __forceinline__ f2 decode(f2 v, int) const { return v; }
@@ -65,7 +64,7 @@ __global__ void __launch_bounds__(kResMaxWarps * 32, 1) resident_batch_kernel(co
         k.lut = a.lut;
         k.fields = nullptr;
         k.ffirst = k.fevery = n;
-        resident_run<BASIS, SAMPLE>(k, ReplicaPar<SAMPLE>{KeyPairs(h.cc.key), h.pc, h, (double)h.gram_s}, res_smem + kResHotBytes);
+        resident_run<BASIS, SAMPLE>(k, ReplicaPar<SAMPLE>{KeyPairs(h.cc.key), h.pc, h, SAMPLE == kResExact ? 1.0 : (double)h.gram_s}, res_smem + kResHotBytes);
     }
     // the last CTA to finish advances the batch step (every CTA read it at its start)
     if (threadIdx.x == 0) {

@@ -1,0 +1,58 @@
+"""Correlation sums with FP32 products (batches in the 128x4 and 64x8 shapes) against FP64 sums of the very states they sampled, so that nothing but the
+rounding of the sums themselves is left.
+
+Products of FP32 numbers are added up in FP32, rounded to nearest, in chains of
+at most K = 260 (a lane's share of a warp's 1024 nodes, and two more sums), then in
+FP64. A chain's partial sums grow to its total, so a chain is off by about
+sqrt(K / 3) 2^-24 / sqrt(3) of it, without bias, and the sum of M chains by that over
+sqrt(M). With K / M below 1 / 200 in each case here, four of these are
+4 / 3 sqrt(1 / 200) 2^-24 < 2^-27; the bound is twice that, of sqrt(S2_ii S2_jj). (Sums
+that cut off instead of rounding are 2^-24 too small and more.)"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1204_6734_gb300 import flb, inputs
+
+pytestmark = pytest.mark.gpu
+
+BOUND = 2.0 ** -26
+
+
+def params(Lx, Ly, r=0, precision="fp32", basis="local", kT=1e-4):
+    return inputs.LatticeParams(Lx, Ly, 1.0, 0.1, 0.02, kT, inputs.omega_groups(1.2, 0.9, 1.0), basis, precision,
+                                seed=30 + r, replica=r)
+
+
+def check(S1, S2, n, states, p):
+    # the kernels subtract c = f^0(rho0, u0) as FP32 numbers
+    c = oracle.init_equilibrium(p)[:, :1, 0].astype(np.float32).astype(np.float64)
+    R1, R2, m = np.zeros(9), np.zeros((9, 9)), 0
+    for f in states:
+        d = f.reshape(9, -1) - c
+        R1 += d.sum(1)
+        R2 += d @ d.T
+        m += d.shape[1]
+    assert n == m
+    q = np.sqrt(np.diag(R2))
+    assert np.abs((S2 - R2) / np.outer(q, q)).max() <= BOUND
+    assert np.abs((S1 - R1) / (q * np.sqrt(n))).max() <= BOUND
+
+
+@pytest.mark.parametrize("shapes,kinds", [([(21, 21)] * 24, {"resident"}), ([(9, 7)] * 200, {"resident"}),
+                                          ([(64, 64)] * 8, {"cut"}), ([(300, 48)] * 2, {"cut"})])
+@pytest.mark.parametrize("tile", ["128x4", "64x8"])
+@pytest.mark.parametrize("kT", [1e-4, 1e-3])
+def test_batches(shapes, kinds, tile, kT):
+    ps = [params(Lx, Ly, r, kT=kT) for r, (Lx, Ly) in enumerate(shapes)]
+    n = 40
+    with flb.Batch(ps, tile=tile) as b, flb.Batch(ps, tile=tile, kernel="pipelined") as w:
+        b.set_sampling(0, 1)
+        b.step(n)
+        assert b.launches()[0] == kinds
+        sums = [b.raw_sums(r) for r in range(len(ps))]
+        states = []
+        for _ in range(n):
+            states += [w.populations(r) for r in range(len(ps))]
+            w.step(1)
+    check(sum(s[0] for s in sums), sum(s[1] for s in sums), sum(s[2] for s in sums), states, ps[0])
