@@ -557,7 +557,7 @@ cudaError_t launch_resident(flb_lattice h, int n, float* fields) {
     if (half) {   // the codec of launch_step_fp16
         const DevCodec c = dev_codec(h);
         a.scale = c.scale;
-        a.s = c.scale;
+        a.s = 1.0;
         a.sinv = 1.0f / c.scale;
         for (int i = 0; i < 9; ++i) a.snref[i] = -c.ref[i] * a.sinv;
     }
@@ -613,9 +613,9 @@ cudaError_t launch_step(flb_lattice h, bool sample, float* fields = nullptr) {
 // The resident launch of a lattice, if it ever pays.
 ResidentPlan plan_resident(const flb_params* p, int sms, bool cut) {
     if (p->precision == FLB_FP64) return ResidentPlan();
-    const ResidentPlan r = resident_plan(p->Lx, p->Ly, sms, cut);
     const double nodes = (double)p->Lx * p->Ly;
     const bool half = p->precision == FLB_FP16_DEV;
+    const ResidentPlan r = resident_plan(p->Lx, p->Ly, sms, cut, half);
     return resident_pays(r, nodes, half, false) || resident_pays(r, nodes, half, true) ? r : ResidentPlan();
 }
 

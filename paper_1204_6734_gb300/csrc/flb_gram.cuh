@@ -87,12 +87,6 @@ __device__ __forceinline__ void gram_store(uint32_t st, f2 h) {
                  "r"(*reinterpret_cast<const uint32_t*>(&v)));
 }
 
-template <int I>
-__device__ __forceinline__ void gram_store_raw(uint32_t st, __half2 v) {
-    asm volatile("st.shared.b32 [%0+%1], %2;" ::"r"(st), "n"(2 * kGramRowHalves * I),
-                 "r"(*reinterpret_cast<const uint32_t*>(&v)));
-}
-
 template <int S>
 __device__ __forceinline__ void gram_step(uint32_t ld, float (&c)[8]) {
     uint32_t d0, d1, d2, d3;
@@ -119,20 +113,6 @@ __device__ __forceinline__ void gram_stage(const GramLane& g, const f2 (&h)[9]) 
     gram_store<8>(g.st, h[8]);
 }
 
-// The same from values that are FP16 already.
-__device__ __forceinline__ void gram_stage_raw(const GramLane& g, const __half2 (&h)[9]) {
-    __syncwarp();
-    gram_store_raw<0>(g.st, h[0]);
-    gram_store_raw<1>(g.st, h[1]);
-    gram_store_raw<2>(g.st, h[2]);
-    gram_store_raw<3>(g.st, h[3]);
-    gram_store_raw<4>(g.st, h[4]);
-    gram_store_raw<5>(g.st, h[5]);
-    gram_store_raw<6>(g.st, h[6]);
-    gram_store_raw<7>(g.st, h[7]);
-    gram_store_raw<8>(g.st, h[8]);
-}
-
 // Add the staged block to c: four 16-node steps of two mma.m16n8k16 each.
 __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
     __syncwarp();
@@ -140,29 +120,6 @@ __device__ __forceinline__ void gram_mma(const GramLane& g, float (&c)[8]) {
     gram_step<1>(g.ld, c);
     gram_step<2>(g.ld, c);
     gram_step<3>(g.ld, c);
-}
-
-// As gram_mma, with every 16 nodes' sums started from zero and added to c outside
-// the tensor cores, rounded to nearest (their accumulators cut off): for values
-// that are FP16 numbers to begin with, whose products FP32 holds exactly.
-// Every 16 nodes rather than every 64: <df df> of 2000 x 1500 against FP64 7.0e-7
-// rather than 8.0e-7 (the FP32 products these sums replaced: 7.0e-7), the step 63.8
-// us rather than 63.2.
-template <int S>
-__device__ __forceinline__ void gram_step_rn(uint32_t ld, float (&c)[8]) {
-    float p[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) p[q] = 0.f;
-    gram_step<S>(ld, p);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) c[q] += p[q];
-}
-__device__ __forceinline__ void gram_mma_rn(const GramLane& g, float (&c)[8]) {
-    __syncwarp();
-    gram_step_rn<0>(g.ld, c);
-    gram_step_rn<1>(g.ld, c);
-    gram_step_rn<2>(g.ld, c);
-    gram_step_rn<3>(g.ld, c);
 }
 
 // Add the FP32 partials to the FP64 matrix cm[16][16] (rows and columns 0..9
@@ -195,15 +152,17 @@ __device__ __forceinline__ double gram_sum(const double* cm, int q, double s) {
 
 // ---------------------------------------------------------------------------
 // The same sums with FP32 products, rounded to nearest throughout: for batches in
-// the tile shapes that promise them.
+// the tile shapes that promise them, and for the FP16 store, whose values are FP16
+// numbers to begin with (their products are exact).
 //
 // A warp stages its 64 nodes in FP32 (rows 0..8, row 9 ones). The ten rows make
 // five pairs, the upper triangle of their products 15 blocks of 2 x 2 entries, and
 // two lanes share a block, each with every other four nodes: 32 128-bit loads and
 // 64 packed multiply-adds per 64 nodes, four packed sums per lane across tiles.
 // Rows are 68 floats apart, so that the lanes of a load meet two banks twice at
-// most. Tensor cores cut off where this rounds: with deviations in two FP16 halves in
-// place of FP32 products <df df> was 2e-7 too small.
+// most. Tensor cores cut off where this rounds: <df df> of the FP16 store was
+// 4.7e-8 too small with them, and 2e-7 with deviations in two FP16 halves in place
+// of FP32 products (6e-10 with products added up by sampler warps).
 // ---------------------------------------------------------------------------
 constexpr int kProdRowFloats = 68;                        // 64 nodes + 4 floats
 constexpr int kProdWarpFloats = 10 * kProdRowFloats;      // one warp's block: 2720 bytes

@@ -11,17 +11,17 @@ namespace flb {
 
 namespace {
 
-template <class Par>
+template <class Par, int SAMPLE>
 const void* kernel_of(int basis, bool sample) {
     if (basis == 0)
-        return sample ? (const void*)resident_kernel<0, kResStaged, Par> : (const void*)resident_kernel<0, kResQuiet, Par>;
+        return sample ? (const void*)resident_kernel<0, SAMPLE, Par> : (const void*)resident_kernel<0, kResQuiet, Par>;
     if (basis == 1)
-        return sample ? (const void*)resident_kernel<1, kResStaged, Par> : (const void*)resident_kernel<1, kResQuiet, Par>;
-    return sample ? (const void*)resident_kernel<2, kResStaged, Par> : (const void*)resident_kernel<2, kResQuiet, Par>;
+        return sample ? (const void*)resident_kernel<1, SAMPLE, Par> : (const void*)resident_kernel<1, kResQuiet, Par>;
+    return sample ? (const void*)resident_kernel<2, SAMPLE, Par> : (const void*)resident_kernel<2, kResQuiet, Par>;
 }
 
 const void* kernel_of(int basis, bool half, bool sample) {
-    return half ? kernel_of<LatticePar16>(basis, sample) : kernel_of<LatticePar>(basis, sample);
+    return half ? kernel_of<LatticePar16, kResExact>(basis, sample) : kernel_of<LatticePar, kResStaged>(basis, sample);
 }
 
 }  // namespace
@@ -58,7 +58,7 @@ bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample) 
     return sample ? 1.12 * us + 0.3 < (half ? 5.9 : 7.9) + rest : us + 0.6 < (half ? 3.4 : 4.0) + rest;
 }
 
-ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
+ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut, bool half) {
     ResidentPlan best;
     if (36LL * Lx * Ly > (long long)(cut ? sms : 1) * (long long)kResSmemMax) return best;
     double cost = 1e30;
@@ -74,7 +74,7 @@ ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut) {
             // sampling: three more warps, if there is room, for the reduction
             const int swarps = std::min(kResMaxWarps, wp + 3);
             const size_t q = res_smem_bytes((int)cells, kResQuiet, warps);
-            const size_t t = res_smem_bytes((int)cells, kResStaged, swarps);
+            const size_t t = res_smem_bytes((int)cells, half ? kResExact : kResStaged, swarps);
             if (q > kResSmemMax) continue;
             const double c = resident_step_us(wp, gx, gy, bw, bh);
             if (c >= cost) continue;

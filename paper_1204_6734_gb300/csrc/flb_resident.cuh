@@ -42,7 +42,8 @@
 // resident at once (cooperative launch), every wait is bounded (flb_tma.cuh).
 //
 // Correlation sums: as flb_gram.cuh (staged in FP16 for the tensor cores, or with
-// FP32 products where a batch's tile shape promises them), except that every step's FP32 partials (at most 1024 products per warp, added
+// FP32 products where a batch's tile shape promises them and for the FP16 store),
+// except that every step's FP32 partials (at most 1024 products per warp, added
 // over the CTA's warps in FP32 in a fixed order) go to FP64 by themselves: the sums
 // do not depend on how many steps a launch makes.
 #pragma once
@@ -563,8 +564,6 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
                 if (smp) {
                     if constexpr (kExact)
                         prod_sums(gp, reinterpret_cast<float(&)[8]>(gc));
-                    else if constexpr (sizeof(Store) == 2)
-                        gram_mma_rn(gh, reinterpret_cast<float(&)[8]>(gc));
                     else
                         gram_mma(gh, reinterpret_cast<float(&)[8]>(gc));
                 }
@@ -653,7 +652,7 @@ struct LatticePar16 {
     const CollideConst<float>& cc;
     const ResidentArgs& a;
     double s;
-    __device__ __forceinline__ f2 scaled(f2 v, int) const { return v; }
+    __device__ __forceinline__ f2 scaled(f2 v, int) const { return v * f2(a.scale); }
     __device__ __forceinline__ float ref(int i) const { return a.ref[i]; }
     __device__ __forceinline__ f2 decode(f2 v, int i) const { return mad(v, f2(a.scale), f2(a.ref[i])); }
     __device__ __forceinline__ f2 encode(f2 f, int i) const {
@@ -704,7 +703,7 @@ double resident_step_us(int wp, int gx, int gy, int bw, int bh);
 // Whether a launch of many steps is faster than one launch per step.
 bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample);
 // Cut a lattice for the given number of SMs; `cut` = false: one block only.
-ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut);
+ResidentPlan resident_plan(int Lx, int Ly, int sms, bool cut, bool half);
 // Raise the kernels' dynamic shared memory limit (once per plan).
 cudaError_t resident_prepare(const ResidentPlan& p, int basis, bool half);
 cudaError_t resident_step(const ResidentPlan& p, const ResidentArgs& a, const CollideConst<float>& cc, int basis,

@@ -14,10 +14,12 @@
 // refilling it. Boxes start 8 columns left of the tile (a TMA box of 16-bit
 // elements must start at a multiple of 8 elements) and are 144 wide.
 //
-// Correlation sums on the tensor cores (flb_gram.cuh): h is the deviation from c
-// and an FP16 number already, so it is staged as it was read and the products
-// are exact. Sampler warps (4 beside 8 colliding warps) formed the same products
-// in FP32 registers: 94.4 us per step at 2000 x 1500, f-norm, against 65.6 with 16 warps here.
+// Correlation sums with FP32 products by the colliding warps (flb_gram.cuh) of the
+// deviations sqrt(kT) h, rounded to FP32. (Squares of h itself, exact in FP32, end in
+// one of few bit patterns, and their sums rounded to nearest came out 3e-8 to 8e-8
+// too small.) Sampler warps (4 beside 8 colliding warps) formed the same products in
+// FP32 registers: 94.4 us per step at 2000 x 1500, f-norm, against 65.4 here; on the
+// tensor cores they took 63.8, 4.7e-8 of <df df> lost to their cut-off.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -44,8 +46,8 @@ struct HShape {
     static constexpr int STAGE = 9 * SPLANE;       // halves per stage (10.4 / 20.7 KB)
     static constexpr int STAGES = NW == 8 ? 16 : 9;
     static constexpr size_t smem_bytes() {
-        return sizeof(__half) * (size_t)STAGES * STAGE + 2 * STAGES * sizeof(uint64_t) + sizeof(double) * 256 +
-               sizeof(__half) * (size_t)NW * kGramWarpHalves;
+        return sizeof(__half) * (size_t)STAGES * STAGE + 2 * STAGES * sizeof(uint64_t) + sizeof(double) * 64 +
+               sizeof(float) * (size_t)NW * kProdWarpFloats;
     }
     static_assert((SPLANE * sizeof(__half)) % 128 == 0, "plane boxes stay 128-byte aligned");
     static_assert((NW & (NW - 1)) == 0, "release counts wrap at 2^32");
@@ -73,8 +75,8 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
     __half* smem = reinterpret_cast<__half*>(smem_raw);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * HS::STAGE);
     uint32_t* released = reinterpret_cast<uint32_t*>(full + S);   // releases of each stage
-    double* red = reinterpret_cast<double*>(full + 2 * S);        // FP64 Gram matrix (16 x 16)
-    __half* gram = reinterpret_cast<__half*>(red + 256);
+    double* red = reinterpret_cast<double*>(full + 2 * S);        // FP64 sums (kProdEntries)
+    float* staged = reinterpret_cast<float*>(red + 64);
 
     const int c = threadIdx.x, warp = c >> 5, lane_id = c & 31;
     allow_dependents();
@@ -86,8 +88,8 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
         fence_mbar_init();
     }
     if constexpr (SAMPLE) {
-        for (int q = c; q < 256; q += NW * 32) red[q] = 0.0;
-        gram_init(gram + warp * kGramWarpHalves);
+        if (c < kProdEntries) red[c] = 0.0;
+        prod_init(staged + warp * kProdWarpFloats);
     }
     __syncthreads();
     wait_dependency();
@@ -101,7 +103,7 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
             issue_tile16<NW>(smem, &map, a, t, j, full);
     }
     const int ty = c >> 6, r = c & 63;
-    const GramLane gblk(SAMPLE ? smem_u32(gram + warp * kGramWarpHalves) : 0u, kGramRows);
+    const ProdLane gblk(SAMPLE ? smem_u32(staged + warp * kProdWarpFloats) : 0u);
     float gc[SAMPLE ? 8 : 1];
     if constexpr (SAMPLE) {
 #pragma unroll
@@ -123,15 +125,12 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
                 h[i] = __halves2half2(p[0], p[64]);
             }
         };
-        auto decode = [&](const __half2* h, f2* g) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) g[i] = mad(f2(__half22float2(h[i])), f2(a.scale), f2(a.ref[i]));
-        };
         f2 g[9];
         {
             __half2 h[9];
             raw(h);
-            decode(h, g);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) g[i] = mad(f2(__half22float2(h[i])), f2(a.scale), f2(a.ref[i]));
         }
         const int tty = t / a.tiles_x, x0 = (t - tty * a.tiles_x) * kTW, y0 = tty * TH, y = y0 + ty;
         const int xA = x0 + r, xB = xA + 64;
@@ -140,15 +139,19 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
         auto refetch = [&](f2* gg) {
             __half2 h[9];
             raw(h);
-            decode(h, gg);
-            if constexpr (SAMPLE) {
-                if (!whole) {
-                    const __half z = __float2half_rn(0.f);
+            f2 v[9];
 #pragma unroll
-                    for (int i = 0; i < 9; ++i)
-                        h[i] = __halves2half2(inA ? __low2half(h[i]) : z, inB ? __high2half(h[i]) : z);
+            for (int i = 0; i < 9; ++i) {
+                v[i] = f2(__half22float2(h[i]));
+                gg[i] = mad(v[i], f2(a.scale), f2(a.ref[i]));
+            }
+            if constexpr (SAMPLE) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    v[i] = v[i] * f2(a.scale);
+                    if (!whole) v[i] = f2(inA ? v[i].v.x : 0.f, inB ? v[i].v.y : 0.f);
                 }
-                gram_stage_raw(gblk, h);
+                prod_stage(gblk, v);
             }
         };
         const uint32_t nodeA = a.node0 + (uint32_t)xA + (uint32_t)Lx * (uint32_t)y;
@@ -156,9 +159,9 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
         const uint32_t stt = collide_basis<f2, BASIS>(g, PairNoise{cc.key, nodeA, nodeA + 64u, a.step}, refetch, a.lut,
                                                       cc, f);
         if constexpr (SAMPLE) {
-            gram_mma_rn(gblk, reinterpret_cast<float(&)[8]>(gc));
+            prod_sums(gblk, reinterpret_cast<float(&)[8]>(gc));
             if (++gtiles == kGramFlushTiles) {
-                gram_flush(reinterpret_cast<float(&)[8]>(gc), red);
+                prod_flush(reinterpret_cast<float(&)[8]>(gc), red);
                 gtiles = 0;
             }
         }
@@ -207,9 +210,9 @@ step_fp16_kernel(const __grid_constant__ CUtensorMap map, const HArgs a, const C
             if (!mbar_wait(&full[j % S], (j / S) & 1)) break;
     }
     if constexpr (SAMPLE) {
-        gram_flush(reinterpret_cast<float(&)[8]>(gc), red);
+        prod_flush(reinterpret_cast<float(&)[8]>(gc), red);
         __syncthreads();
-        if (c < kSums) atomicAdd(&a.acc[c], gram_sum(red, c, (double)a.scale));
+        if (c < kSums) atomicAdd(&a.acc[c], prod_sum(red, c, 1.0));
     }
 }
 

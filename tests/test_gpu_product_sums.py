@@ -1,4 +1,5 @@
-"""Correlation sums with FP32 products (batches in the 128x4 and 64x8 shapes) against FP64 sums of the very states they sampled, so that nothing but the
+"""Correlation sums with FP32 products (batches in the 128x4 and 64x8 shapes, the FP16
+store) against FP64 sums of the very states they sampled, so that nothing but the
 rounding of the sums themselves is left.
 
 Products of FP32 numbers are added up in FP32, rounded to nearest, in chains of
@@ -56,3 +57,22 @@ def test_batches(shapes, kinds, tile, kT):
             states += [w.populations(r) for r in range(len(ps))]
             w.step(1)
     check(sum(s[0] for s in sums), sum(s[1] for s in sums), sum(s[2] for s in sums), states, ps[0])
+
+
+@pytest.mark.parametrize("Lx,Ly,n,kinds", [(21, 21, 500, {"resident"}), (300, 130, 30, {"cut"}), (257, 129, 30, {"cut"}),
+                                           (900, 900, 4, {"step"}), (2000, 700, 2, {"step"})])
+@pytest.mark.parametrize("basis", ["local", "standard", "lut"])
+def test_fp16_store(Lx, Ly, n, kinds, basis):
+    p = params(Lx, Ly, precision="fp16dev", basis=basis)
+    with flb.Lattice(p) as lat, flb.Lattice(p) as w:
+        w.step(3)
+        lat.step(3)
+        lat.set_sampling(3, 1)
+        assert lat.step(n).launches()[0] == kinds
+        S1, S2, m = lat.raw_sums()
+
+        def states():
+            for _ in range(n):
+                yield w.populations()
+                w.step(1)
+        check(S1, S2, m, states(), p)
