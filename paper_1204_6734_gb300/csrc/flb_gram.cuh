@@ -152,8 +152,7 @@ __device__ __forceinline__ double gram_sum(const double* cm, int q, double s) {
 
 // ---------------------------------------------------------------------------
 // The same sums with FP32 products, rounded to nearest throughout: for batches in
-// the tile shapes that promise them, and for the FP16 store, whose values are FP16
-// numbers to begin with (their products are exact).
+// the tile shapes that promise them, and for the FP16 store.
 //
 // A warp stages its 64 nodes in FP32 (rows 0..8, row 9 ones). The ten rows make
 // five pairs, the upper triangle of their products 15 blocks of 2 x 2 entries, and

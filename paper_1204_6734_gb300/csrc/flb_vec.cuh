@@ -89,4 +89,11 @@ __device__ __forceinline__ float lane(f2 a, int k) { return k ? a.v.y : a.v.x; }
 template <class V> struct Elem { using type = V; };
 template <> struct Elem<f2> { using type = float; };
 
+// a + b, its rounding error (exact: Knuth, TAOCP 2, 4.2.2) added to lo.
+__device__ __forceinline__ float two_sum(float a, float b, float& lo) {
+    const float t = a + b, z = t - a;
+    lo += (a - (t - z)) + (b - z);
+    return t;
+}
+
 }  // namespace flb

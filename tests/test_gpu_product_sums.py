@@ -76,3 +76,30 @@ def test_fp16_store(Lx, Ly, n, kinds, basis):
                 yield w.populations()
                 w.step(1)
         check(S1, S2, m, states(), p)
+
+
+@pytest.mark.parametrize("shapes,kinds", [([(21, 21)] * 3, {"resident"}), ([(30, 30)] * 700, {"resident"}),
+                                          ([(64, 64)] * 8, {"cut"}), ([(300, 130)], {"cut"})])
+def test_partials_of_the_warps_meet_in_fp64(shapes, kinds):
+    """Deviations k 2^-25, 2^15 <= k < 2^16, from populations that are powers of two: the
+    sum of the 256 nodes that a warp takes at most here is exact in FP32, that of all
+    warps is not, so S1 is exact only if the warps' partials are added in FP64 (or as
+    it would)."""
+    ps = [inputs.LatticeParams(Lx, Ly, 36 / 64, 0.0, 0.0, 1e-4, inputs.omega_groups(1.2, 0.9, 1.0), "local", "fp32",
+                               seed=r, replica=r) for r, (Lx, Ly) in enumerate(shapes)]
+    c = np.array([16] + [4] * 4 + [1] * 4)[:, None] / 64   # f^0 of rho = 36 / 64 at rest
+    g = np.random.Generator(np.random.PCG64(4))
+    with flb.Batch(ps) as b:
+        want = {}
+        for r in (0, len(ps) - 1):
+            p = ps[r]
+            d = g.integers(2 ** 15, 2 ** 16, (9, p.nodes)) * 2.0 ** -25
+            b.set_populations(r, (c + d).reshape(9, p.Ly, p.Lx))
+            want[r] = d.sum(1)
+        b.set_sampling(0, 1000)
+        b.step(4)
+        assert b.launches()[0] == kinds
+        for r, s in want.items():
+            S1, _, n = b.raw_sums(r)
+            assert n == ps[r].nodes
+            np.testing.assert_array_equal(S1, s)
