@@ -127,9 +127,10 @@ int flb_sync(flb_lattice h);
 int flb_time(flb_lattice h, int64_t* t);
 
 /* Checkpoint and resume. A run continues exactly (the same noise draws, the
- * same sampling schedule, the same sums up to FP64 rounding order --
- * up to the rounding of the FP32 partials (FLB_OPT_PIPELINE_SAMPLING 3) where an
- * FP32 run mixes calls of one or two steps with longer ones) from its
+ * same sampling schedule, the same sums up to FP64 rounding order, however the
+ * steps are cut into calls; up to the rounding of FP32 partials of at most 1024
+ * products between handles with and without a workspace of the caller's, and
+ * for steps that the caller captures, which other kernels may take) from its
  * state f_i(x, t) (flb_get_populations), its time t (flb_time) and its raw
  * sums (flb_raw_sums): on a new handle with the same parameters call
  * flb_set_sampling (which clears the sums), then flb_set_raw_sums,

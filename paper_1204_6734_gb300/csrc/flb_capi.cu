@@ -493,18 +493,20 @@ DevCodec dev_codec(flb_lattice h) {
 
 // How many of the next n steps one resident launch takes (0: none): the kernel
 // is on, the lattice fits, and the stream is not being captured (a mailbox tag
-// may not be replayed). The steps before the first sampled one go by themselves
-// (the kernel without sampling) where that leaves no short launch.
+// may not be replayed). A sampled step takes it in calls of any length, so that the
+// sums do not depend on how a run is cut into calls; fewer than kResMinSteps steps
+// without samples go one by one. The steps before the first sampled one go by
+// themselves (the kernel without sampling) where there are enough of them.
 int64_t resident_steps(flb_lattice h, int64_t n) {
-    if (!h->res.gx || h->variant != FLB_KERNEL_AUTO || h->one_step || h->slab) return 0;
-    if (n < kResMinSteps) return 0;
+    if (!h->res.gx || h->variant != FLB_KERNEL_AUTO || h->one_step || h->slab || n < 1) return 0;
     n = resident_launch_steps(n, h->res.us);
     if (h->every > 0 && h->t < h->warmup) {
         const int64_t quiet = h->warmup - h->t;
-        if (quiet >= kResMinSteps && n - quiet >= kResMinSteps) n = quiet;
+        if (quiet >= kResMinSteps && n > quiet) n = quiet;
     }
     const bool sample = count_sampled(h->t, h->t + n, h->warmup, h->every) > 0;
-    if (!resident_pays(h->res, (double)h->p.Lx * h->p.Ly, h->p.precision == FLB_FP16_DEV, sample) ||
+    if ((!sample && n < kResMinSteps) ||
+        !resident_pays(h->res, (double)h->p.Lx * h->p.Ly, h->p.precision == FLB_FP16_DEV, sample) ||
         (sample && h->p.precision == FLB_FP32 && h->tma.sample_mode != kPlanTensorSampling))
         return 0;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
