@@ -30,28 +30,34 @@ const void* kernel_of(int basis, bool half, bool sample) {
 // nodes on the four schedulers of an SM; blocks that exchange add their words'
 // trip through L2 and the passes whose lanes move them (a row on the edge; a
 // block of one row waits at both). A cut across x puts edge lanes into every
-// row, and a warp waits at one edge after the other. Measured: 21 x 21 in one
-// block 1.8, in two 2.1; 64 x 64 in 1 / 4 / 16 / 64 blocks 11.1 / 3.4 / 2.0 / 2.7;
-// 300 x 130 in 26 / 44 / 65 / 130 blocks 5.2 / 3.7 / 3.5 / 4.1, in 2 x 65 4.7, 3 x 43
-// 7.1; 626 x 62 in 1 x 62 4.7, 2 x 62 4.4, 2 x 31 5.5, 7 x 21 7.3; 4000 x 20 in 2 / 4 / 7
-// x 20 10.5 / 5.7 / 5.0; 512 x 512 in 128 blocks 7.0, 2 x 74 7.1; 1000 x 750 in 150
-// 16.4. Sampling adds 0.4 (21 x 21) to 2.7 (1000 x 750).
-// (Taken before the cells' byte addresses and the edges' scalar arguments, which
-// made a step 3 to 9 % faster: 21 x 21 sampled 2.0, 300 x 130 sampled 4.0, 1000 x 750
-// 15.0; the other cuts were not timed again.)
+// row, and a warp waits at one edge after the other: blocks of five rows and more
+// lose 9 us, and narrow ones 1.4 us in every pass of a scheduler that holds an edge.
+// Measured: 21 x 21 in one block 1.6; 64 x 64 in 1 / 4 / 16 / 64 blocks 11.1 / 3.4 /
+// 2.0 / 2.7; 300 x 130 in 26 / 44 / 65 / 130 blocks 5.2 / 3.7 / 3.4 / 4.1, in 2 x 65 4.7,
+// 3 x 43 7.1; 626 x 62 in 1 x 62 4.7, 2 x 62 4.4, 2 x 31 5.5, 7 x 21 7.3; 4000 x 20 in
+// 2 / 4 / 7 x 20 10.5 / 5.7 / 5.0; 512 x 512 in 128 blocks 6.5; 593 x 1269 in 141 15.1; 1000 x
+// 750 in 150 15.0 (large blocks come out up to a tenth faster than estimated).
+// Sampled, across x: 5000 x 100 in 152 x 1 28.9, 3000 x 150 in 75 x 2 23.4, 1648 x 176 in
+// 50 x 3 17.3, 2923 x 132 in 38 x 4 16.0, 1147 x 319 in 36 x 4 22.3 and in 10 x 15 16.7 (one
+// launch per step: 16.2, 14.6, 12.4, 14.4, 14.3).
 double resident_step_us(int wp, int gx, int gy, int bw, int bh) {
-    double t = std::max(1.75, 0.69 * ((wp + 3) / 4) + 0.3);
+    const int passes = (wp + 3) / 4;
+    double t = std::max(1.75, 0.69 * passes + 0.3);
     if (gy > 1) t += 0.3 + 0.072 * bw / 32.0 + (bh == 1 ? 1.2 : 0.0);   // one row: two waits in a row
-    if (gx > 1) t += bh == 1 ? 0.3 : bh == 2 ? 2.3 : 5.0;
+    if (gx > 1)
+        t += std::max(bh == 1 ? 0.3 : bh == 2 ? 2.3 : bh < 5 ? 5.0 : 9.0, 1.4 * passes * std::min(1.0, 40.0 / bw));
     return t;
 }
 
-// One launch per step, without / with sampling, measured: FP32 up to 300 x 130
-// 4.0 / 8.0, 400 x 300 6.4 / 10.0, 512 x 512 8.5 / 12.0, 700 x 600 10.3 / 14.2, 1000 x
-// 750 17.8 / 20.5, 900 x 900 19.4 / 22.6; FP16 store 3.4 / 5.9, 5.2 / 7.7, 8.5 / 11.0,
-// 11.0 / 14.2, 15.5 / 20.3, 18.0 / 22.6. Against that this kernel: 300 x 130 3.5 / 4.1,
-// 626 x 62 4.4 / 5.3, 400 x 300 4.2 / 4.9, 512 x 512 7.0 / 8.0, 700 x 600 9.5 / 10.9,
-// 1000 x 750 16.3 / 19.1, 900 x 900 17.6 / 20.7; the FP16 store 3 to 5 % more.
+// us per step without / with sampling, this kernel and one launch per step: f-norm
+// 21 x 21 1.6 / 2.1 and 4.0 / 6.7, 300 x 130 3.3 / 4.0 and 4.0 / 8.1, 400 x 300 4.0 / 4.8
+// and 6.4 / 10.2, 512 x 512 6.5 / 7.7 and 8.5 / 12.2, 700 x 600 8.9 / 10.4 and 10.3 / 14.3,
+// 1000 x 750 15.0 / 17.5 and 17.9 / 20.8, 900 x 900 16.3 / 19.0 and 19.4 / 22.9; the Hermite
+// norm 300 x 130 2.6 / 3.1 and 2.8 / 7.3, 512 x 512 4.6 / 5.4 and 5.9 / 10.0, 900 x 900 10.9 /
+// 13.0 and 14.4 / 17.0; the FP16 store 300 x 130 3.3 / 4.2 and 3.2 / 5.1, 512 x 512 6.6 / 9.1
+// and 8.3 / 10.8, 700 x 600 9.0 / 11.8 and 10.8 / 14.4. Of 90 shapes drawn up to 1.15
+// million nodes, in the f-norm and the Hermite norm, five took longer here: 1066 x 153,
+// sampled, by 8 %, and four without sampling in the Hermite norm (about 3 us) by 2 to 17 %.
 bool resident_pays(const ResidentPlan& p, double nodes, bool half, bool sample) {
     if (!p.gx || !p.smem[sample]) return false;
     const double us = half ? 1.05 * p.us : p.us, rest = nodes / 54e3;
