@@ -141,7 +141,8 @@ int flb_time(flb_lattice h, int64_t* t);
 int flb_set_time(flb_lattice h, int64_t t);
 int flb_set_raw_sums(flb_lattice h, const double* S1, const double* S2, int64_t n_samples);
 
-/* Node and step of the first recorded device error (-1, -1 if none). */
+/* Node and step of the first recorded device error (-1, -1 if none): of the
+ * earliest step that had one. */
 int flb_error_location(flb_lattice h, int64_t* node, int64_t* step);
 
 /* Forget a recorded device error (the state is left as it is). */

@@ -22,7 +22,7 @@ constexpr int kStepThreads = 256;
 
 struct DevError {
     int code;        // 0 = none, else kStatus*
-    int pad;
+    int lock;        // record_earliest
     long long node;
     long long step;
 };
@@ -50,6 +50,38 @@ __device__ __forceinline__ void record_error(DevError* err, int code, long long 
         err->node = node;
         err->step = step;
     }
+}
+
+// Whether an error at (step, node) comes before the recorded one, both from a launch
+// of the steps t0 .. t0 + n - 1 (32-bit step counters); one recorded by an earlier
+// launch stays.
+__host__ __device__ inline bool error_precedes(const DevError& had, long long node, uint32_t step, uint32_t t0, int n) {
+    if (had.code == 0) return true;
+    const uint32_t a = (uint32_t)had.step - t0, b = step - t0;
+    if (a >= (uint32_t)n) return false;
+    return b < a || (b == a && node < had.node);
+}
+
+// Record the earliest error of a launch whose blocks may be several steps apart:
+// one thread per block at a time (the lock is held for a few reads and writes by a
+// thread that runs; it is not waited for without end).
+static __device__ __noinline__ void record_earliest(DevError* err, int code, long long node, uint32_t step, uint32_t t0, int n) {
+    int tries = 0;
+    while (atomicCAS(&err->lock, 0, 1) != 0)
+        if (++tries == 1 << 16) return record_error(err, code, node, step);
+    __threadfence();
+    volatile DevError* e = err;
+    DevError had;
+    had.code = e->code;
+    had.node = e->node;
+    had.step = e->step;
+    if (error_precedes(had, node, step, t0, n)) {
+        e->node = node;
+        e->step = step;
+        e->code = code;
+    }
+    __threadfence();
+    atomicExch(&err->lock, 0);
 }
 
 // Accumulation type of the per-thread correlation sums: FP32 for the FP32

@@ -218,7 +218,7 @@ __device__ __forceinline__ void store_cells(const ResCells& a, const f2 (&f)[9],
 template <int AXIS, int I0, int I1, int I2>
 __device__ __noinline__ void res_receive(const uint64_t* in, uint32_t tag, int g, int j, int n, int first, int u, int v,
                                          uint32_t a0, uint32_t a1, uint32_t a2, uint32_t b0, uint32_t b1, uint32_t b2,
-                                         bool skip1, bool skip2, volatile int* gave_up, DevError* err, uint32_t t) {
+                                         bool skip1, bool skip2, volatile int* gave_up) {
     const ResAxis ax{g, j, n, first};
     const uint64_t* pa0 = in + res_word<AXIS, I0, true>(ax, u);
     const uint64_t* pa1 = in + res_word<AXIS, I1, true>(ax, u);
@@ -247,7 +247,7 @@ __device__ __noinline__ void res_receive(const uint64_t* in, uint32_t tag, int g
         if (began == 0) {
             began = clock64();
         } else if (clock64() - began > kWaitCycles) {
-            record_error(err, kStatusTimeout, -1, t);
+            gave_up[1] = (int)tag;
             *gave_up = 1;
             break;
         }
@@ -283,11 +283,9 @@ __device__ __noinline__ void res_send(uint64_t* out, uint32_t tag, int g, int j,
 // The calls for one edge of a pair.
 template <int AXIS, int I0, int I1, int I2>
 __device__ __forceinline__ void res_edge_in(const uint64_t* in, uint32_t tag, const ResAxis& ax, int u, int v,
-                                            const ResCells& a, bool skip1, bool skip2, volatile int* gave_up,
-                                            DevError* err, uint32_t t) {
+                                            const ResCells& a, bool skip1, bool skip2, volatile int* gave_up) {
     res_receive<AXIS, I0, I1, I2>(in, tag, ax.g, ax.j, ax.n, ax.first, u, v, a.a<I0>(), a.a<I1>(), a.a<I2>(),
-                                  a.b<opposite(I0)>(), a.b<opposite(I1)>(), a.b<opposite(I2)>(), skip1, skip2, gave_up,
-                                  err, t);
+                                  a.b<opposite(I0)>(), a.b<opposite(I1)>(), a.b<opposite(I2)>(), skip1, skip2, gave_up);
 }
 template <int AXIS, int I0, int I1, int I2>
 __device__ __forceinline__ void res_edge_out(uint64_t* out, uint32_t tag, const ResAxis& ax, int u, int v,
@@ -374,9 +372,14 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
     double* red = reinterpret_cast<double*>(after);
     float* slots = reinterpret_cast<float*>(after + (SAMPLE ? kResSlot * 8 : 0));
     __half* gram = reinterpret_cast<__half*>(slots + (SAMPLE ? 2 * nw * kResSlot : 0));
-    volatile int* gave_up =
-        reinterpret_cast<volatile int*>(after + res_sample_bytes(SAMPLE, nw));
-    if (c == 0) *gave_up = 0;
+    // {a wait gave up, its tag}, then the block's first error: step of the launch, node,
+    // code (kStatusNonfinite: 1)
+    volatile int* gave_up = reinterpret_cast<volatile int*>(after + res_sample_bytes(SAMPLE, nw));
+    const auto first_error = [&] { return reinterpret_cast<unsigned long long*>(const_cast<int*>(gave_up) + 2); };
+    if (c == 0) {
+        *gave_up = 0;
+        *first_error() = ~0ull;
+    }
 
     constexpr bool kExact = SAMPLE == kResExact;
     const uint32_t blk = SAMPLE ? smem_u32(gram) + warp * (kExact ? kProdWarpFloats * 4 : kGramWarpHalves * 2) : 0u;
@@ -423,6 +426,8 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
             }
         }
     }
+
+    __syncthreads();
 
     // in bytes: a row of cells, all cells; the steps between a thread's pairs; the
     // steps so far modulo the block
@@ -481,10 +486,10 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
                 const uint32_t tag = k.tag0 + (uint32_t)st;
                 int X, Y, XB, YB;
                 place(X, Y, XB, YB);
-                if (e.b) res_edge_in<1, 2, 5, 6>(in, tag, ay, X, XB, a, false, false, gave_up, k.err, t);
-                if (e.t) res_edge_in<1, 4, 7, 8>(in, tag, ay, X, XB, a, false, false, gave_up, k.err, t);
-                if (e.l) res_edge_in<0, 1, 5, 8>(in, tag, ax, Y, YB, a, e.b, e.t, gave_up, k.err, t);
-                if (e.r) res_edge_in<0, 3, 7, 6>(in, tag, ax, Y, YB, a, e.t, e.b, gave_up, k.err, t);
+                if (e.b) res_edge_in<1, 2, 5, 6>(in, tag, ay, X, XB, a, false, false, gave_up);
+                if (e.t) res_edge_in<1, 4, 7, 8>(in, tag, ay, X, XB, a, false, false, gave_up);
+                if (e.l) res_edge_in<0, 1, 5, 8>(in, tag, ax, Y, YB, a, e.b, e.t, gave_up);
+                if (e.r) res_edge_in<0, 3, 7, 6>(in, tag, ax, Y, YB, a, e.t, e.b, gave_up);
             }
             auto load = [&](f2(&g)[9]) {
                 if (inA) {
@@ -545,8 +550,9 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
             const uint32_t stt =
                 collide_basis<f2, BASIS>(g, PairNoiseT<typename Par::Key>{par.key, nodeA, nodeB, t}, refetch, k.lut, par.cc, f);
             if (stt) {
-                if (inA && (stt & 0xFF)) record_error(k.err, (int)(stt & 0xFF), nodeA, t);
-                if (inB && (stt >> 8)) record_error(k.err, (int)(stt >> 8), nodeB, t);
+                const unsigned long long at = (unsigned long long)st << 32;   // nodes are below 2^31
+                if (inA && (stt & 0xFF)) atomicMin(first_error(), at | nodeA << 1 | ((stt & 0xFF) == kStatusNonfinite));
+                if (inB && (stt >> 8)) atomicMin(first_error(), at | nodeB << 1 | ((stt >> 8) == kStatusNonfinite));
             }
 #pragma unroll
             for (int i = 0; i < 9; ++i) f[i] = par.encode(f[i], i);
@@ -598,8 +604,15 @@ __device__ __forceinline__ void resident_run_of(const ResBlock& k, const Par& pa
         sy = sy + row == all ? 0u : sy + row;
         if (!last) __syncthreads();
     }
+    __syncthreads();
+    if (c == 0) {
+        const unsigned long long e = *first_error();
+        if (e != ~0ull)
+            record_earliest(k.err, e & 1 ? kStatusNonfinite : kStatusInvalidVelocity, (uint32_t)e >> 1,
+                            k.t0 + (uint32_t)(e >> 32), k.t0, k.n);
+        if (*gave_up) record_earliest(k.err, kStatusTimeout, -1, k.t0 + ((uint32_t)gave_up[1] - k.tag0), k.t0, k.n);
+    }
     if constexpr (SAMPLE != kResQuiet) {
-        __syncthreads();
         if (pending) res_reduce<SAMPLE>(slots + ((nsum - 1) & 1) * nw * kResSlot, red, nwork);
         __syncthreads();
         if (nsum)

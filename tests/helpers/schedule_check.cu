@@ -4,3 +4,12 @@
 extern "C" long long sampled(long long ta, long long tb, long long warmup, long long every) {
     return flb::count_sampled(ta, tb, warmup, every);
 }
+
+// Whether an error at (step, node) of a launch of n steps from t0 replaces a recorded one.
+extern "C" int precedes(int code, long long had_node, long long had_step, long long node, unsigned step, unsigned t0, int n) {
+    flb::DevError had{};
+    had.code = code;
+    had.node = had_node;
+    had.step = had_step;
+    return flb::error_precedes(had, node, step, t0, n);
+}
