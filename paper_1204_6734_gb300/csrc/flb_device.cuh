@@ -76,17 +76,27 @@ __device__ __forceinline__ void draw_fields(const Draw& d, uint32_t k[6]) {
 
 // Box-Muller: u1 = (k_{2p}+1) 2^-21 in (0,1], u2 = k_{2p+1} 2^-21 in [0,1),
 // N_{2p} = sqrt(-2 ln u1) cos(2 pi u2), N_{2p+1} = sqrt(-2 ln u1) sin(2 pi u2).
+// In FP64 the radius and the first quarter of the circle come from these two
+// functions, at the node or from tables that were filled by them (flb_step64.cuh):
+// the normals are the same bits either way.
+constexpr int kQuarter = 1 << 19;   // angles of 2^-21 turns in a quarter
+__device__ __forceinline__ double bm_radius(uint32_t k) { return sqrt(-2.0 * log(((double)k + 1.0) * 0x1p-21)); }
+__device__ __forceinline__ double2 bm_circle(uint32_t j) {   // j < kQuarter
+    double s, c;
+    sincospi((double)j * 0x1p-20, &s, &c);
+    return make_double2(c, s);
+}
+// Radius r and point e of the first quarter, turned by q quarters: (c, s), (-s, c),
+// (-c, -s), (s, -c).
+__device__ __forceinline__ void bm_pair(double r, double2 e, uint32_t q, double* n) {
+    const double x = r * ((q & 1) ? e.y : e.x), y = r * ((q & 1) ? e.x : e.y);
+    n[0] = (q == 1 || q == 2) ? -x : x;
+    n[1] = q >= 2 ? -y : y;
+}
 __device__ __forceinline__ void box_muller(const uint32_t k[6], double n[6]) {
 #pragma unroll
-    for (int p = 0; p < 3; ++p) {
-        const double u1 = ((double)k[2 * p] + 1.0) * 0x1p-21;
-        const double u2 = (double)k[2 * p + 1] * 0x1p-21;
-        const double r = sqrt(-2.0 * log(u1));
-        double s, c;
-        sincos(kTwoPi * u2, &s, &c);
-        n[2 * p] = r * c;
-        n[2 * p + 1] = r * s;
-    }
+    for (int p = 0; p < 3; ++p)
+        bm_pair(bm_radius(k[2 * p]), bm_circle(k[2 * p + 1] & (kQuarter - 1)), k[2 * p + 1] >> 19, n + 2 * p);
 }
 
 // FP32 form with the SFU: ln u1 = ln2 * log2(u1) (MUFU.LG2, absolute error

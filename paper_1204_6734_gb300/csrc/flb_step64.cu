@@ -2,13 +2,14 @@
 // per block, pulled, sampled, collided and stored.
 //
 // Bound: the FP64 pipe (two lanes a cycle and SM). The collision and the sums
-// are about 450 FP64 operations per node, and until now the noise, six divided
-// square roots and the block's reduction were another 600; so:
+// are about 450 FP64 operations per node; the noise by functions, six divided
+// square roots and the block's reduction by shuffles would be another 600; so:
 //  * Normals by table. A draw has 21-bit fields: the radius sqrt(-2 ln u1) has
 //    2^21 values, cosine and sine 2^19 up to signs and their exchange. Both come
 //    from tables in L2 (16.8 and 8.4 MB; three 8-byte and three 16-byte reads
-//    per node), computed once by the very functions that the kernel called
-//    for every node (three logarithms, square roots and sine-cosine pairs).
+//    per node), computed once by the functions that would be called for every
+//    node (bm_radius and bm_circle, flb_device.cuh: three logarithms, square
+//    roots and sine-cosine pairs); without tables they are.
 //  * 1 / sqrt(pivot) as rsqrt (flb_vec.cuh).
 //  * The 54 sums of a warp by folding: in every round a lane keeps half of its
 //    values and adds its partner's share of them, 62 additions in place of 270.
@@ -31,17 +32,12 @@ namespace flb {
 
 namespace {
 
-// The radius and (cosine, sine) of box_muller (flb_device.cuh): entry k of the
-// radius table is that of the field k; entry j of the circle that of angle
-// 2 pi j 2^-21.
+// Entry k of the radius table is that of the field k; entry j of the circle that of
+// the angle 2 pi j 2^-21.
 __global__ void noise_tables_kernel(double* radius, double2* circle) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < kRadius) radius[k] = sqrt(-2.0 * log(((double)k + 1.0) * 0x1p-21));
-    if (k < kQuarter) {
-        double s, c;
-        sincospi((double)k * 0x1p-20, &s, &c);
-        circle[k] = make_double2(c, s);
-    }
+    if (k < kRadius) radius[k] = bm_radius(k);
+    if (k < kQuarter) circle[k] = bm_circle(k);
 }
 
 // The warp's totals of s[0..53]: lane l gets sums 2 l and 2 l + 1.

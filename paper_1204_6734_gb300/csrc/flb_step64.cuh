@@ -10,7 +10,8 @@ namespace flb {
 // Device tables of the FP64 noise on the current device, built on first use
 // and kept until the process exits (25 MB): the Box-Muller radius of each of
 // the 2^21 values of u1, and cosine and sine of the first quarter of the 2^21
-// angles. Null where there is no memory for them.
+// angles. Null where there is no memory for them (the kernels then form the same
+// numbers themselves).
 struct NoiseTables {
     const double* radius = nullptr;
     const double2* circle = nullptr;
@@ -18,7 +19,6 @@ struct NoiseTables {
 NoiseTables noise_tables();
 
 constexpr int kRadius = 1 << 21;
-constexpr int kQuarter = 1 << 19;
 
 // A node's normals from the tables (unit normals of NodeNoise in FP64).
 struct TableNoise {
@@ -28,16 +28,13 @@ struct TableNoise {
     __device__ __forceinline__ void operator()(double n[6]) const {
         uint32_t k[6];
         node_fields(key, node, step, k);
+        of(tab, k, n);
+    }
+    static __device__ __forceinline__ void of(const NoiseTables& tab, const uint32_t k[6], double n[6]) {
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const double r = __ldg(tab.radius + k[2 * p]);
-            const uint32_t q = k[2 * p + 1] >> 19;   // quarter: (c, s), (-s, c), (-c, -s), (s, -c)
-            const double2 e = __ldg(tab.circle + (k[2 * p + 1] & (kQuarter - 1)));
-            const double c = (q & 1) ? e.y : e.x, s = (q & 1) ? e.x : e.y;
-            const double x = r * c, y = r * s;
-            n[2 * p] = (q == 1 || q == 2) ? -x : x;
-            n[2 * p + 1] = q >= 2 ? -y : y;
-        }
+        for (int p = 0; p < 3; ++p)
+            bm_pair(__ldg(tab.radius + k[2 * p]), __ldg(tab.circle + (k[2 * p + 1] & (kQuarter - 1))), k[2 * p + 1] >> 19,
+                    n + 2 * p);
     }
 };
 
