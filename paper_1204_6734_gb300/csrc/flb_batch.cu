@@ -514,15 +514,17 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     // blocks exchanges 96 bytes per column, a node is 72 bytes of the pool)
     const size_t rtab_bytes = Arena::round_up(sizeof(ResCta) * std::max(max_replicas, b->sms));
     const size_t mail_bytes = Arena::round_up(std::min<size_t>(pool_bytes / 4, 16u << 20));
-    const size_t meta_bytes = desc_bytes + tile_bytes + ctl_bytes + acc_bytes + err_bytes + rtab_bytes + mail_bytes +
-                              Arena::round_up(sizeof(double) * kFinalizeOut);
+    const size_t scratch_bytes = Arena::round_up(sizeof(double) * kFinalizeOut);
+    size_t meta_bytes = desc_bytes + tile_bytes + ctl_bytes + acc_bytes + err_bytes + rtab_bytes + scratch_bytes;
     void *pool = nullptr, *meta = nullptr;
-    if (cudaMalloc(&pool, pool_bytes) != cudaSuccess || cudaMalloc(&meta, meta_bytes) != cudaSuccess) {
-        cudaGetLastError();
+    bool mailboxes = false;   // without them no replica is cut
+    if (device_alloc(&pool, pool_bytes) != cudaSuccess ||
+        alloc_with_extra(device_alloc, &meta, meta_bytes, mail_bytes, &mailboxes) != cudaSuccess) {
         if (pool) cudaFree(pool);
         delete b;
         return FLB_ERR_OOM;
     }
+    if (mailboxes) meta_bytes += mail_bytes;
     b->pool = (char*)pool;
     b->arena.reset(pool_bytes);
     b->meta = (char*)meta;
@@ -539,10 +541,10 @@ int flb_batch_open(int32_t basis, int32_t max_replicas, size_t pool_bytes, void*
     m += err_bytes;
     b->rtable = (ResCta*)m;
     m += rtab_bytes;
-    b->mail = (uint64_t*)m;
-    m += mail_bytes;
     b->scratch = (double*)m;
-    b->mail_words = mail_bytes / sizeof(uint64_t);
+    m += scratch_bytes;
+    b->mail = mailboxes ? (uint64_t*)m : nullptr;
+    b->mail_words = mailboxes ? mail_bytes / sizeof(uint64_t) : 0;
 
     ce = cudaMemsetAsync(b->meta, 0, meta_bytes, b->stream);
     if (ce == cudaSuccess && b->basis == FLB_BASIS_LOCAL_LUT && lut_tables(&b->lut, nullptr) != FLB_OK)

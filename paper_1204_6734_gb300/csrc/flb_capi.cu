@@ -663,16 +663,12 @@ int lattice_create(const flb_params* p, void* dev_workspace, size_t workspace_by
         h->res = plan_resident(p, sms, true);
         const size_t mail = 2 * sizeof(uint64_t) * (size_t)h->res.mail_words;
         void* ptr = nullptr;
-        if (mail && cudaMalloc(&ptr, L.total + mail) != cudaSuccess) {
-            cudaGetLastError();
-            ptr = nullptr;
-            h->res = plan_resident(p, sms, false);
-        }
-        if (!ptr && cudaMalloc(&ptr, L.total) != cudaSuccess) {
-            cudaGetLastError();
+        bool mailboxes = false;
+        if (alloc_with_extra(device_alloc, &ptr, L.total, mail, &mailboxes) != cudaSuccess) {
             delete h;
             return FLB_ERR_OOM;
         }
+        if (!mailboxes) h->res = plan_resident(p, sms, false);
         h->ws = (char*)ptr;
         h->own_ws = true;
         if (h->res.mail_words) {

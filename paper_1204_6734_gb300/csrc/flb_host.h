@@ -124,6 +124,27 @@ inline bool tensor_sampling_ok(const flb_params* p) {
 }
 inline double gram_scale(const flb_params* p) { return std::sqrt(p->kT * p->rho0); }
 
+// Allocate need + extra bytes or, where they cannot be had, need; *got_extra tells
+// which. alloc(&p, bytes): cudaMalloc.
+template <class Alloc>
+cudaError_t alloc_with_extra(Alloc&& alloc, void** p, size_t need, size_t extra, bool* got_extra) {
+    *p = nullptr;
+    *got_extra = true;
+    cudaError_t ce = alloc(p, need + extra);
+    if (ce != cudaSuccess && extra > 0) {
+        *p = nullptr;
+        *got_extra = false;
+        ce = alloc(p, need);
+    }
+    return ce;
+}
+// cudaMalloc, its error not left behind.
+inline cudaError_t device_alloc(void** p, size_t bytes) {
+    const cudaError_t ce = cudaMalloc(p, bytes);
+    if (ce != cudaSuccess) cudaGetLastError();
+    return ce;
+}
+
 // Steps of [ta, tb) that the schedule (warmup, every) samples. No sum of times
 // passes tb or warmup, so any `every` up to 2^63 - 1 will do.
 inline int64_t count_sampled(int64_t ta, int64_t tb, int64_t warmup, int64_t every) {

@@ -13,3 +13,20 @@ extern "C" int precedes(int code, long long had_node, long long had_step, long l
     had.step = had_step;
     return flb::error_precedes(had, node, step, t0, n);
 }
+
+// alloc_with_extra over a device with `free` bytes: the bytes it got (-1: an error), and
+// whether the extra ones are among them.
+extern "C" long long extra(long long free, long long need, long long extra_bytes, int* got) {
+    void* p;
+    bool with = false;
+    long long bytes = -1;
+    const auto alloc = [&](void** q, size_t n) {
+        if ((long long)n > free) return cudaErrorMemoryAllocation;
+        bytes = (long long)n;
+        *q = &bytes;
+        return cudaSuccess;
+    };
+    const cudaError_t ce = flb::alloc_with_extra(alloc, &p, (size_t)need, (size_t)extra_bytes, &with);
+    *got = with;
+    return ce == cudaSuccess && p ? bytes : -1;
+}
