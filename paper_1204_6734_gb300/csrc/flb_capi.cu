@@ -333,7 +333,7 @@ struct flb_lattice_s {
     double* pending64 = nullptr;   // partial sums of the last FP64 step, not yet in acc
     NoiseTables noise;   // FP64 lattices
     double* acc;         // kSums running sums
-    double* small;       // basis (81) + finalize output (171) + conservation (3)
+    double* small;       // finalize output (kFinalizeOut), conservation (3), partial sums
     DevError* err;
     cudaStream_t stream;
     int64_t t, warmup, every, nsamp;
@@ -402,7 +402,7 @@ Layout layout(const flb_params* p, int sms) {
     L.acc_off = off;
     off += align_up(sizeof(double) * kSums);
     L.small_off = off;
-    off += align_up(sizeof(double) * (81 + 171 + 3 + 3 * (size_t)L.nblocks));
+    off += align_up(sizeof(double) * (kFinalizeOut + 3 + 3 * (size_t)L.nblocks));
     L.err_off = off;
     off += align_up(sizeof(DevError));
     L.total = off;
@@ -415,7 +415,7 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? FLB_OK : FLB_ERR_CUDA; }
 // The generic FP32 kernel (one node per thread, plain loads).
 template <int BASIS, bool SAMPLE>
 cudaError_t launch_generic_t(flb_lattice h) {
-    StepArgs<float> a;
+    StepArgs a;
     a.src = (const float*)h->buf[h->cur];
     a.dst = (float*)h->buf[h->cur ^ 1];
     a.geo = h->geo;
@@ -425,7 +425,7 @@ cudaError_t launch_generic_t(flb_lattice h) {
     a.err = h->err;
     a.lut = h->lut32;
     for (int i = 0; i < 9; ++i) a.ref[i] = (float)h->ref[i];
-    step_kernel<float, BASIS, SAMPLE><<<h->nblocks, kStepThreads, 0, h->stream>>>(a, collide_const<float>(&h->p));
+    step_kernel<BASIS, SAMPLE><<<h->nblocks, kStepThreads, 0, h->stream>>>(a, collide_const<float>(&h->p));
     return cudaGetLastError();
 }
 
@@ -1129,7 +1129,7 @@ int flb_correlations(flb_lattice h, int32_t measure_basis, double* Cff, double* 
     if (rc) return rc;
     if (n_samples) *n_samples = h->nsamp;
     if (h->nsamp <= 0) return FLB_ERR_STATE;
-    double* res = h->small + 81;
+    double* res = h->small;
     finalize_kernel<<<1, kFinalizeThreads, 0, h->stream>>>(h->acc, h->nsamp, measure_basis, h->p.ux0, h->p.uy0, res);
     double host[171];
     cudaError_t ce = cudaGetLastError();
@@ -1145,8 +1145,8 @@ int flb_correlations(flb_lattice h, int32_t measure_basis, double* Cff, double* 
 
 int flb_conservation(flb_lattice h, double sums[3]) {
     if (!h || !sums) return FLB_ERR_ARG;
-    double* part = h->small + 81 + 171 + 3;
-    double* res = h->small + 81 + 171;
+    double* part = h->small + kFinalizeOut + 3;
+    double* res = h->small + kFinalizeOut;
     if (h->p.precision == FLB_FP64)
         conservation_kernel<double><<<h->nblocks, kStepThreads, 0, h->stream>>>(
             (const double*)h->buf[h->cur], h->geo, part, DevCodec());

@@ -31,17 +31,16 @@ struct Vec9 {
     double v[9];
 };
 
-template <class T>
 struct StepArgs {
-    const T* src;
-    T* dst;
+    const float* src;
+    float* dst;
     Geometry geo;
     uint32_t step;
     uint32_t node0;     // noise counter of node (0, 0): Lx y0 for a slab starting at row y0
     double* partials;   // [gridDim.x][kSums] when sampling
     DevError* err;
-    const T* lut;       // velocity table (look-up-table f-norm only)
-    T ref[9];           // c = f^0(rho0, u0), subtracted before sampling
+    const float* lut;   // velocity table (look-up-table f-norm only)
+    float ref[9];       // c = f^0(rho0, u0), subtracted before sampling
 };
 
 __device__ __forceinline__ void record_error(DevError* err, int code, long long node,
@@ -84,12 +83,8 @@ static __device__ __noinline__ void record_earliest(DevError* err, int code, lon
     atomicExch(&err->lock, 0);
 }
 
-// Accumulation type of the per-thread correlation sums: FP32 for the FP32
-// path (a thread sums a few hundred nodes at most), FP64 otherwise; per-block
-// partials and everything after them are FP64.
-template <class T>
-struct AccType { using type = T; };
-
+// Per-block sums of the per-thread ones (FP32 on the FP32 path: a thread sums a few
+// hundred nodes at most), added over the warps in FP64.
 template <class A>
 __device__ __forceinline__ void block_reduce_sums(A (&s)[kSums], double* out) {
     __shared__ double red[kStepThreads / 32][kSums];
@@ -109,29 +104,28 @@ __device__ __forceinline__ void block_reduce_sums(A (&s)[kSums], double* out) {
     }
 }
 
-// Fused step: pull-stream, (sample), collide with noise, store.
-template <class T, int BASIS, bool SAMPLE>
+// Fused FP32 step, one node per thread: pull-stream, (sample), collide with noise, store.
+template <int BASIS, bool SAMPLE>
 __global__ void __launch_bounds__(kStepThreads)
-step_kernel(StepArgs<T> a, CollideConst<T> cc) {
-    using A = typename AccType<T>::type;
+step_kernel(StepArgs a, CollideConst<float> cc) {
     const int Lx = a.geo.Lx;
     const long long N = (long long)Lx * a.geo.Ly;
-    A s[kSums];
+    float s[kSums];
     if (SAMPLE) {
 #pragma unroll
-        for (int k = 0; k < kSums; ++k) s[k] = A(0);
+        for (int k = 0; k < kSums; ++k) s[k] = 0.f;
     }
     // N < 2^31 (checked at creation): 32-bit node indices
     for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < (int)N; n += gridDim.x * blockDim.x) {
         const int y = n / Lx;
         const int x = n - y * Lx;
-        T g[9];
+        float g[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) g[i] = a.src[at(a.geo, i, x - cvx(i), y - cvy(i))];
         if (SAMPLE) {
-            A d[9];
+            float d[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) d[i] = A(g[i]) - A(a.ref[i]);
+            for (int i = 0; i < 9; ++i) d[i] = g[i] - a.ref[i];
             int k = 9;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
@@ -140,10 +134,10 @@ step_kernel(StepArgs<T> a, CollideConst<T> cc) {
                 for (int j = i; j < 9; ++j) s[k++] += d[i] * d[j];
             }
         }
-        T f[9];
-        const uint32_t st = collide_basis<T, BASIS>(
+        float f[9];
+        const uint32_t st = collide_basis<float, BASIS>(
             g, NodeNoise{cc.key, a.node0 + (uint32_t)n, a.step},
-            [&](T* gg) {
+            [&](float* gg) {
 #pragma unroll
                 for (int i = 0; i < 9; ++i) gg[i] = g[i];
             },
@@ -151,7 +145,7 @@ step_kernel(StepArgs<T> a, CollideConst<T> cc) {
         if (st != kStatusOk) record_error(a.err, (int)(st & 0xFF), (long long)a.node0 + n, a.step);
         store_node(a.dst, a.geo, x, y, f);
     }
-    if (SAMPLE) block_reduce_sums<A>(s, a.partials + (long long)blockIdx.x * kSums);
+    if (SAMPLE) block_reduce_sums<float>(s, a.partials + (long long)blockIdx.x * kSums);
 }
 
 // Sum over blocks of partials[b * kSums + q], computed by one warp: lane l adds
