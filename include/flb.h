@@ -99,6 +99,13 @@ size_t flb_workspace_bytes(const flb_params* p);
  *                 least flb_workspace_bytes(p) bytes, 256-byte aligned, that the
  *                 caller keeps alive until flb_destroy.
  *  stream:        a cudaStream_t (as void*), or NULL for the default stream.
+ * Beside the workspace, the first FP64 lattice of a CUDA context makes the library
+ * allocate 25 MB of noise tables there, and the first lattice in the look-up-table
+ * f-norm its velocity tables; both stay until the process exits. Without memory for
+ * the noise tables the kernels form the same numbers themselves, more slowly. A
+ * library-owned allocation also holds the exchange buffers of lattices that flb_step
+ * cuts into blocks (see FLB_OPT_KERNEL); without room for them, and on a caller's
+ * workspace, such lattices take one launch per step.
  * Errors: FLB_ERR_ARG (parameters), FLB_ERR_OOM, FLB_ERR_CUDA. */
 int flb_create(const flb_params* p, void* dev_workspace, size_t workspace_bytes,
                void* stream, flb_lattice* out);
@@ -116,7 +123,9 @@ int flb_set_sampling(flb_lattice h, int64_t warmup, int64_t every);
 int flb_reset_statistics(flb_lattice h);
 
 /* Enqueue n time steps of Eq. LBE1 (pull streaming, collision with noise) on
- * the handle's stream; returns without waiting. Errors: FLB_ERR_ARG (n < 0),
+ * the handle's stream; returns without waiting. Small and middling FP32 and
+ * FP16_DEV lattices make many steps per launch (FLB_OPT_KERNEL); such a launch
+ * holds its SMs for about 10 ms at most. Errors: FLB_ERR_ARG (n < 0),
  * a recorded device error (sticky), FLB_ERR_CUDA. */
 int flb_step(flb_lattice h, int64_t n);
 
@@ -261,7 +270,8 @@ int flb_collide_nodes(const flb_params* p, const double* g, const uint32_t* node
 /* ---------------------------------------------------------------------------
  * Batches: many independent FP32 lattices ("replicas") of different sizes and
  * parameters, stepped together by one persistent launch per step of the
- * pipelined kernel (the tiles of all replicas in one table). Each replica has
+ * pipelined kernel (the tiles of all replicas in one table) or, where they fit the
+ * SMs' shared memory, by launches of many steps. Each replica has
  * its own state, noise stream (its seed and replica id), time, sampling
  * schedule and sums, and error record; its populations are those of a lattice
  * handle created with the same parameters and stepped as often, and its sums
@@ -282,8 +292,9 @@ typedef struct flb_batch_s* flb_batch;
  * 128 x 4 nodes, 2 nodes per thread (default);
  * 64 x 8 nodes, 2 nodes per thread (wastes less on narrow lattices);
  * 128 x 2 nodes, 1 node per thread;
- *   (these three: 8 colliding warps per CTA beside 4 sampler warps on
- *   sampling steps, FP32 products)
+ *   (these three form the sums from FP32 products: in single-step launches by 4
+ *   sampler warps beside 8 colliding warps per CTA, in launches of many steps by the
+ *   colliding warps)
  * 128 x 6 and 64 x 12 nodes, 2 nodes per thread, 12 colliding warps that add
  *   their own nodes to the correlation sums on the tensor cores (deviations
  *   staged in FP16, as FLB_OPT_PIPELINE_SAMPLING 3 of a lattice): only when
@@ -420,8 +431,9 @@ int flb_batch_set_populations(flb_batch b, int32_t slot, const double* host_in);
  * The host enqueues work up to two chunks of `chunk_steps` steps ahead of the
  * GPU. Like batches, this has no counterpart in the paper.
  *
- * Modes: FLB_SERVE_BATCHED runs all admitted requests as one batch (one
- * launch per step, chunks replayed from a CUDA graph); FLB_SERVE_PER_LATTICE
+ * Modes: FLB_SERVE_BATCHED runs all admitted requests as one batch, a chunk at a
+ * time (flb_batch_step: in one launch where the running requests allow it, else one
+ * launch per step replayed from a CUDA graph); FLB_SERVE_PER_LATTICE
  * gives each its own lattice handle (one launch per lattice and step), for
  * comparison. A request's result does not depend on the mode or on the other
  * requests, up to the summation order of its sums.
@@ -482,12 +494,13 @@ int flb_server_stats(flb_server s, flb_serve_stats* out);
 int flb_server_set_tile(flb_server s, int32_t tile);
 
 /* Tuning and testing options of a lattice handle.
- *  FLB_OPT_KERNEL: which step kernel runs -- FLB_KERNEL_AUTO (default: for FP32
- *    the pipelined TMA kernel, or, in calls of three steps or more on lattices
- *    that fit the SMs' shared memory, a kernel that makes all of them in one
- *    launch; the generic kernel for FP64),
- *    FLB_KERNEL_GENERIC (one node per thread, plain loads) or
- *    FLB_KERNEL_PIPELINED (FP32 only). All give the same results up to rounding.
+ *  FLB_OPT_KERNEL: which step kernel runs -- FLB_KERNEL_AUTO (default): for FP32
+ *    and the FP16 store a kernel that keeps the populations in shared memory and
+ *    makes many steps per launch, on lattices that fit it and are faster that way
+ *    (sampled steps in calls of any length, others in calls of three steps or more),
+ *    the pipelined TMA kernel otherwise; FLB_KERNEL_GENERIC (FP32 only: one node per
+ *    thread, plain loads); FLB_KERNEL_PIPELINED (FP32 only). FP64 has one kernel and
+ *    takes AUTO and GENERIC alike. All give the same results up to rounding.
  *  FLB_OPT_PIPELINE_WARPS: colliding warps per CTA of the pipelined kernel
  *    (8, 12, 14 or 16; the tile is 128 x value/2 nodes) for every step. By
  *    default the f-norm bases use 16 on lattices of at least 8 such tiles

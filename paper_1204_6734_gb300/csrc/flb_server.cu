@@ -6,8 +6,8 @@
 // device pool (the HBM budget) are free. Admitted requests run together:
 //
 //  * batched mode: all running requests are replicas of one batch
-//    (flb_batch.cu), stepped by one persistent launch per step, in chunks of
-//    `chunk` steps replayed from a CUDA graph;
+//    (flb_batch.cu), stepped in chunks of `chunk` steps: one launch where the
+//    requests allow it, else one per step replayed from a CUDA graph;
 //  * per-lattice mode (the comparison): each running request is its own
 //    lattice handle on a workspace carved from the same pool, stepped by one
 //    launch per lattice and step.

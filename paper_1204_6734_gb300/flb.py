@@ -733,7 +733,7 @@ class Lattice:
 
 
 class Batch:
-    """Many FP32 lattices stepped by one launch per step (owns an flb_batch).
+    """Many FP32 lattices stepped together (owns an flb_batch).
 
     ``Batch(params_list)`` adds the given lattices as slots 0..n-1 with no step
     limit; ``Batch.open(basis, max_replicas, pool_bytes)`` starts empty, for
