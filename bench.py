@@ -28,15 +28,15 @@ sys.path.insert(0, ROOT)
 METRIC = "MLUPS & % of HBM roofline (FP32 vs FP64); batched replica-steps/s, p50/p99"
 UNIT = "MLUPS"
 BYTES_PER_NODE = {"fp32": 72, "fp64": 144}
-# DRAM bytes (read + write) per launch of the FP32 step kernel at 4096^2,
-# f-norm basis, sampling every step (tensor-core sums, 12 colliding warps):
-# ncu dram__bytes_read.sum + dram__bytes_write.sum of one 2048^2 launch of
-# the same kernel (156.0 + 99.7 MB) times the 4x nodes; a full-size capture
-# may take only the launch list. Valid only for the kernel version it was
-# taken on.
-DRAM_TRAFFIC = {("fp32", "local", 4096): 4 * (156.00e6 + 99.70e6),
-                ("fp32", "lut", 4096): 4 * (156.00e6 + 98.73e6)}
-TRAFFIC_SOURCE = "ncu dram bytes of a 2048^2 launch of the same kernel, x 4 (the nodes)"
+# DRAM bytes (read + write) per launch of the FP32 step kernel at 4096^2, sampling
+# every step (tensor-core sums, 16 colliding warps): ncu dram__bytes_read.sum +
+# dram__bytes_write.sum of steps that follow one another, the caches as the step
+# before left them (--cache-control none; one pass): 571.9 + 604.2 MB in the f-norm,
+# which walks its tiles there and back, 614.2 + 603.8 MB in the table f-norm, which
+# does not. Valid only for the kernel version it was taken on.
+DRAM_TRAFFIC = {("fp32", "local", 4096): 571.9e6 + 604.2e6,
+                ("fp32", "lut", 4096): 614.2e6 + 603.8e6}
+TRAFFIC_SOURCE = "ncu dram bytes of a launch of this size, caches as the step before left them"
 # FP64 operations per node-step of the FP64 step kernel (f-norm, sampling
 # every step): 2 DFMA + DADD + DMUL thread instructions counted by ncu on a
 # 2048^2 launch (230 + 79 + 117 per node; the FP64 pipe 88 % busy). The
@@ -654,7 +654,7 @@ def run_sweep(args, rank, world, dist, dev):
 def run_sweep21(args, rank, world, dist, dev):
     """--workload sweep21: the u_x0 sweep on the paper's own 21 x 21 lattice.
     --replicas independent copies per (u_x0, basis), all points of one basis in
-    one batch (all steps of a call in one launch), --steps steps sampled every step after a
+    one batch (many steps per launch), --steps steps sampled every step after a
     tenth; the moment variances of the pooled copies (flb_batch_correlations)
     fitted as in the 4096^2 sweep, in the Hermite norm, the local f-norm and
     the table f-norm (the variant the paper's f-norm numbers come from)."""
