@@ -249,12 +249,13 @@ int warp_passes(int64_t cells) { return (int)(((cells + 1) / 2 + 31) / 32); }
 // Plan the resident launch of the present members, or find that one launch per
 // step is faster (rsmem = 0). Small replicas as they are, several CTAs per SM;
 // or, with fewer replicas than SMs, the SMs dealt out one by one to the replica
-// whose step takes longest, as far as the mailboxes have room. Measured, us per step against one launch per step,
-// f-norm, sampled with FP32 products: 384 x 21^2 6.1 against 61.5 (4.8 / 30.1
-// without sampling), 24 x 21^2 2.5 / 14.4, 1280 x 21^2 16.0 / 169, 300 x 48^2
-// 17.1 / 63.6, 8 x 64^2 (cut) 4.4 / 14.4; two to four CTAs per SM within 1 %. A
-// tile shape's promise holds for its sampling: the
-// shapes with sampler warps form FP32 products, the others stage in FP16.
+// whose step takes longest, as far as the mailboxes have room. Measured, us per step
+// against one launch per step, f-norm, sampled with FP32 products / without sampling:
+// 384 x 21^2 5.4 against 56.9 / 4.1 against 27.4, 24 x 21^2 2.4 / 1.5 (11.1 / 4.9),
+// 1280 x 21^2 14.3 / 10.5 (159.9 / 82.2), 300 x 48^2 15.9 / 11.4 (62.9 / 41.1), 8 x 64^2
+// (cut) 4.3 / 3.0 (11.2 / 4.8); two to four CTAs per SM within 1 %. A tile shape's
+// promise holds for its sampling: the shapes with sampler warps form FP32 products,
+// the others stage in FP16.
 void plan_resident(flb_batch_s* b, bool sample) {
     b->rplan_dirty = false;
     b->rplan_sample = sample;

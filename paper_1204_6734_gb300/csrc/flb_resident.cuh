@@ -23,8 +23,9 @@
 // one addition or subtraction each, and what rarely is asked for (a node's place
 // in the lattice) is divided out where it is. As word indices into an array
 // the same took 16.1 instructions per node against 12.4 in the one-step kernel;
-// us per step before and after: 21 x 21 2.18 / 2.08, 300 x 130 4.27 / 4.13, 1000 x 750
-// 16.4 / 15.7, 384 x 21^2 6.25 / 5.90.
+// us per step with those and with these: 21 x 21 2.18 / 2.08, 300 x 130 4.27 / 4.13, 1000 x
+// 750 16.4 / 15.7, 384 x 21^2 6.25 / 5.90 (with all that this file does by now 2.06, 4.11,
+// 15.1, 5.30).
 //
 // Node pairs (packed FP32x2): node A is the m-th of the block, node B the m-th
 // from its end, i.e. (bw - 1 - x, bh - 1 - y), so B's cells follow from A's
